@@ -165,12 +165,12 @@ def generate_sources():
             e += [f"void launch_schwarz_{nm}(const Pairs& P, const Shells& S, const int* list, int n,",
                   "                          const double* boys, double* Q, cudaStream_t st)",
                   "{",
-                  f"    if (n > 0) schwarz_kernel<Cls_{nm}><<<(n + 127) / 128, 128, 0, st>>>(P, S, list, n, boys, Q);",
+                  f"    schwarz_run<Cls_{nm}>(P, S, list, n, boys, Q, st);",
                   "}",
                   f"void launch_prim_schwarz_{nm}(const Pairs& P, const Shells& S, const int* list, int n,",
                   "                               const double* boys, double* pp, float* qp, float* qg, cudaStream_t st)",
                   "{",
-                  f"    if (n > 0) prim_schwarz_kernel<Cls_{nm}><<<(n + 127) / 128, 128, 0, st>>>(P, S, list, n, boys, pp, qp, qg);",
+                  f"    prim_schwarz_run<Cls_{nm}>(P, S, list, n, boys, pp, qp, qg, st);",
                   "}"]
         e.append("}  // namespace pimd\n")
         p = os.path.join(GEN, f"tu_eri_{nm}.cu")

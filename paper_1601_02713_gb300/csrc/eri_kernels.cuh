@@ -500,113 +500,184 @@ __global__ void __launch_bounds__(128) jk_kernel(Pairs P, Shells S, Reps R_, con
                                                   Gall + off, fxs, false);
 }
 
-// Schwarz factors: Q_ab = sqrt(max over functions of (mn|mn)), one thread per pair
+// Contracted Cartesian block (ab|ab) of the primitive quartets first, first +
+// stride, ... < np * np of one pair (primitive i of the bra, j of the ket at
+// j * np + i), spherical: the recursions and the transform are linear, so the
+// blocks of a pair's threads add up to the whole.
 template <class C>
-__global__ void __launch_bounds__(128) schwarz_kernel(Pairs P, Shells S, const int* __restrict__ list, int n,
-                                                      const double* __restrict__ boys, double* __restrict__ Qout)
+__device__ __forceinline__ void pair_block(const Pairs& P, const double* pp, int ab, const double A[3],
+                                           const double B[3], int np, int first, int last, int stride,
+                                           const double* __restrict__ boys, double* cart)
 {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n) return;
-    const int ab = list[idx];
+    const size_t n = P.n;
+    double acc[C::NE * C::NF];
+#pragma unroll
+    for (int i = 0; i < C::NE * C::NF; i++) acc[i] = 0.0;
+    for (int q = first; q < last; q += stride) {
+        double bra[PP_NERI], ket[PP_NERI];
+#pragma unroll
+        for (int f = 0; f < PP_NERI; f++) {
+            bra[f] = pp[((size_t)f * PIMD_MAXPP + q % np) * n + ab];
+            ket[f] = pp[((size_t)f * PIMD_MAXPP + q / np) * n + ab];
+        }
+        PrimQ<double> g;
+        prim_quartet<double>(bra, ket, g);
+        double F[C::L + 1];
+        boys_eval<C::L>(g.T, boys, g.theta, F);
+        C::template vrr<double>(F, g.PA[0], g.PA[1], g.PA[2], g.WP[0], g.WP[1], g.WP[2], g.QC[0], g.QC[1], g.QC[2],
+                                g.WQ[0], g.WQ[1], g.WQ[2], g.o2p, g.o2pr, g.o2q, g.o2qr, g.o2pq, acc);
+    }
+    constexpr int NCART = ncart(C::LA) * ncart(C::LB) * ncart(C::LC) * ncart(C::LD);
+    double tmp[NCART];
+    C::template hrr<double>(acc, A[0] - B[0], A[1] - B[1], A[2] - B[2], A[0] - B[0], A[1] - B[1], A[2] - B[2], cart);
+    cart_to_sph4<C::LA, C::LB, C::LC, C::LD>(cart, tmp);
+}
+
+// Schwarz factors: Q_ab = sqrt(max over functions of (mn|mn)), one block per
+// pair. The pair's primitive quartets (up to 81) are spread over the block's
+// threads, each with its own contracted block, and only the diagonal elements
+// (mn|mn) are summed over the block. Bound by the latency of one thread's
+// FP64 chain ((dd|dd): about 9000 FMAs per primitive quartet), not by
+// throughput: one thread per pair, as before, ran 81 of them one after
+// another ((dd|dd) of one (H2O)8 bead, 36 pairs: 57 ms).
+// A Fock build of one water molecule (24 functions), most of it this set-up:
+// 91.6 -> 18.9 ms with this kernel and the next.
+// blockDim.x = SCHWARZ_WIDE threads (one primitive quartet each) or one warp.
+constexpr int SCHWARZ_WIDE = 96;
+
+template <class C>
+__global__ void __launch_bounds__(SCHWARZ_WIDE) schwarz_kernel(Pairs P, Shells S, const int* __restrict__ list, int n,
+                                                               const double* __restrict__ boys,
+                                                               double* __restrict__ Qout)
+{
+    constexpr int na = nsph(C::LA), nb = nsph(C::LB);
+    __shared__ double s_diag[SCHWARZ_WIDE / 32][na * nb];
+    const int ab = list[blockIdx.x];
     const int sa = P.sa[ab], sb = P.sb[ab];
-    double sbra_l[PP_NERI][PIMD_MAXPP];
     const int np = P.npp[ab];
-    for (int k = 0; k < np; k++)
-        for (int f = 0; f < PP_NERI; f++) sbra_l[f][k] = P.pp[((size_t)f * PIMD_MAXPP + k) * P.n + ab];
     double A[3], B[3];
 #pragma unroll
     for (int x = 0; x < 3; x++) {
         A[x] = S.xyz[3 * sa + x];
         B[x] = S.xyz[3 * sb + x];
     }
-    constexpr int NCART = ncart(C::LA) * ncart(C::LB) * ncart(C::LC) * ncart(C::LD);
-    double cart[NCART], tmp[NCART];
-    const float qone[PIMD_MAXPP] = {1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f};
-    quartet_cart<C, double>(sbra_l, qone, np, P, ab, A, B, A, B, boys, 0.0f, np * P.npp[ab], np * P.npp[ab], cart);
-    cart_to_sph4<C::LA, C::LB, C::LC, C::LD>(cart, tmp);
-    constexpr int na = nsph(C::LA), nb = nsph(C::LB);
-    double m = 0.0;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    double cart[ncart(C::LA) * ncart(C::LB) * ncart(C::LC) * ncart(C::LD)];
+    const bool work = threadIdx.x < np * np;
+    if (work) pair_block<C>(P, P.pp, ab, A, B, np, threadIdx.x, np * np, blockDim.x, boys, cart);
 #pragma unroll
     for (int i = 0; i < na; i++)
 #pragma unroll
-        for (int j = 0; j < nb; j++) m = fmax(m, fabs(cart[((i * nb + j) * na + i) * nb + j]));
-    Qout[ab] = sqrt(m);
+        for (int j = 0; j < nb; j++) {
+            const double v = work ? cart[((i * nb + j) * na + i) * nb + j] : 0.0;
+            double s = v;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) s_diag[w][i * nb + j] = s;
+        }
+    __syncthreads();
+    if (w == 0) {
+        double m = 0.0;
+        if (lane < na * nb) {
+            double s = 0.0;
+            for (int k = 0; k < nw; k++) s += s_diag[k][lane];
+            m = fmax(m, fabs(s));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (lane == 0) Qout[ab] = sqrt(m);
+    }
+}
+
+template <class C>
+static void schwarz_run(const Pairs& P, const Shells& S, const int* list, int n, const double* boys, double* Q,
+                        cudaStream_t st)
+{
+    // one primitive quartet per thread while the blocks' warps fit the chip's
+    // 608 schedulers a few times over; with more pairs one warp per pair, whose
+    // threads take three each and share one horizontal recursion
+    const int threads = n <= 1024 ? SCHWARZ_WIDE : 32;
+    if (n > 0) schwarz_kernel<C><<<n, threads, 0, st>>>(P, S, list, n, boys, Q);
 }
 
 // Primitive-pair Schwarz factors: for every primitive pair k of shell pair ab
-// (one thread per pair), qp_k = sqrt(max over functions of |(kk|kk)|) with
-// the contraction coefficients included, so that |(ij|kl)| <= qp_i qp_l for
-// any primitive quartet (Cauchy-Schwarz for the two charge distributions).
-// The pair's primitive data are then reordered by descending qp (every field,
-// in place) and qp is stored in that order.
+// (one thread per primitive pair, PSW_PAIRS shell pairs per block; one thread
+// per shell pair, as before, ran its nine one after another: 17 ms for the
+// (dd|dd) pairs of one (H2O)8 bead), qp_k = sqrt(max over functions of
+// |(kk|kk)|) with the contraction coefficients included, so that |(ij|kl)| <=
+// qp_i qp_l for any primitive quartet (Cauchy-Schwarz for the two charge
+// distributions). The pair's primitive data are then reordered by descending
+// qp (every field, in place) and qp is stored in that order.
+constexpr int PSW_PAIRS = 7;   // shell pairs per block: 63 of 64 threads
+
 template <class C>
-__global__ void __launch_bounds__(128) prim_schwarz_kernel(Pairs P, Shells S, const int* __restrict__ list, int n,
-                                                           const double* __restrict__ boys, double* pp, float* qp,
-                                                           float* qg)
+__global__ void __launch_bounds__(64) prim_schwarz_kernel(Pairs P, Shells S, const int* __restrict__ list, int n,
+                                                          const double* __restrict__ boys, double* pp, float* qp,
+                                                          float* qg)
 {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n) return;
-    const int ab = list[idx];
-    const int sa = P.sa[ab], sb = P.sb[ab];
-    const int np = P.npp[ab];
+    __shared__ float s_q[PSW_PAIRS][PIMD_MAXPP];
+    __shared__ int s_perm[PSW_PAIRS][PIMD_MAXPP];
+    const int u = threadIdx.x / PIMD_MAXPP, k = threadIdx.x % PIMD_MAXPP;
+    const int idx = blockIdx.x * PSW_PAIRS + u;
+    const bool mine = u < PSW_PAIRS && idx < n;
     const size_t N = P.n;
-    double A[3], B[3];
+    const int ab = mine ? list[idx] : 0;
+    const int np = mine ? P.npp[ab] : 0;
+    if (k < np) {
+        const int sa = P.sa[ab], sb = P.sb[ab];
+        double A[3], B[3];
 #pragma unroll
-    for (int x = 0; x < 3; x++) {
-        A[x] = S.xyz[3 * sa + x];
-        B[x] = S.xyz[3 * sb + x];
-    }
-    constexpr int na = nsph(C::LA), nb = nsph(C::LB);
-    constexpr int NCART = ncart(C::LA) * ncart(C::LB) * ncart(C::LC) * ncart(C::LD);
-    float q[PIMD_MAXPP];
-    int perm[PIMD_MAXPP];
-    for (int k = 0; k < np; k++) {
-        double v[PP_NERI];
-        for (int f = 0; f < PP_NERI; f++) v[f] = pp[((size_t)f * PIMD_MAXPP + k) * N + ab];
-        double acc[C::NE * C::NF];
-        for (int i = 0; i < C::NE * C::NF; i++) acc[i] = 0.0;
-        PrimQ<double> g;
-        prim_quartet<double>(v, v, g);
-        double F[C::L + 1];
-        boys_eval<C::L>(g.T, boys, g.theta, F);
-        C::template vrr<double>(F, g.PA[0], g.PA[1], g.PA[2], g.WP[0], g.WP[1], g.WP[2], g.QC[0], g.QC[1],
-                                g.QC[2], g.WQ[0], g.WQ[1], g.WQ[2], g.o2p, g.o2pr, g.o2q, g.o2qr, g.o2pq, acc);
-        double cart[NCART], tmp[NCART];
-        C::template hrr<double>(acc, A[0] - B[0], A[1] - B[1], A[2] - B[2], A[0] - B[0], A[1] - B[1], A[2] - B[2],
-                                cart);
-        cart_to_sph4<C::LA, C::LB, C::LC, C::LD>(cart, tmp);
+        for (int x = 0; x < 3; x++) {
+            A[x] = S.xyz[3 * sa + x];
+            B[x] = S.xyz[3 * sb + x];
+        }
+        constexpr int na = nsph(C::LA), nb = nsph(C::LB);
+        double cart[ncart(C::LA) * ncart(C::LB) * ncart(C::LC) * ncart(C::LD)];
+        pair_block<C>(P, pp, ab, A, B, np, k * np + k, k * np + k + 1, 1, boys, cart);
         double m = 0.0;
         for (int i = 0; i < na; i++)
             for (int j = 0; j < nb; j++) m = fmax(m, fabs(cart[((i * nb + j) * na + i) * nb + j]));
         // rounded up so that the float bound stays an upper bound
-        q[k] = __double2float_ru(sqrt(m) * (1.0 + 1e-6));
-        perm[k] = k;
+        s_q[u][k] = __double2float_ru(sqrt(m) * (1.0 + 1e-6));
     }
-    // insertion sort of the primitive pairs, descending qp (stable)
-    for (int k = 1; k < np; k++) {
-        const int pk = perm[k];
-        int j = k - 1;
-        while (j >= 0 && q[perm[j]] < q[pk]) {
-            perm[j + 1] = perm[j];
-            j--;
+    __syncthreads();
+    if (mine && k == 0) {
+        // insertion sort of the primitive pairs, descending qp (stable)
+        int* perm = s_perm[u];
+        const float* q = s_q[u];
+        for (int a = 0; a < np; a++) {
+            int j = a - 1;
+            while (j >= 0 && q[perm[j]] < q[a]) {
+                perm[j + 1] = perm[j];
+                j--;
+            }
+            perm[j + 1] = a;
         }
-        perm[j + 1] = pk;
     }
-    for (int f = 0; f < PP_NF; f++) {
-        double v[PIMD_MAXPP];
-        for (int k = 0; k < np; k++) v[k] = pp[((size_t)f * PIMD_MAXPP + k) * N + ab];
-        for (int k = 0; k < np; k++) pp[((size_t)f * PIMD_MAXPP + k) * N + ab] = v[perm[k]];
+    __syncthreads();
+    double v[PP_NF];
+    if (k < np)
+#pragma unroll
+        for (int f = 0; f < PP_NF; f++) v[f] = pp[((size_t)f * PIMD_MAXPP + s_perm[u][k]) * N + ab];
+    __syncthreads();   // every field is read before any is written
+    if (!mine) return;
+    float q = 0.0f, g = 0.0f;
+    if (k < np) {
+#pragma unroll
+        for (int f = 0; f < PP_NF; f++) pp[((size_t)f * PIMD_MAXPP + k) * N + ab] = v[f];
+        q = s_q[u][s_perm[u][k]];
+        g = q * __double2float_ru(2.0 * sqrt(2.0 * fmax(v[PP_EA], v[PP_EB])));
     }
-    for (int k = 0; k < PIMD_MAXPP; k++) {
-        float g = 0.0f;
-        if (k < np) {
-            const double ea = pp[((size_t)PP_EA * PIMD_MAXPP + k) * N + ab];
-            const double eb = pp[((size_t)PP_EB * PIMD_MAXPP + k) * N + ab];
-            g = q[perm[k]] * __double2float_ru(2.0 * sqrt(2.0 * fmax(ea, eb)));
-        }
-        qp[(size_t)k * N + ab] = k < np ? q[perm[k]] : 0.0f;
-        qg[(size_t)k * N + ab] = g;
-    }
+    qp[(size_t)k * N + ab] = q;
+    qg[(size_t)k * N + ab] = g;
+}
+
+template <class C>
+static void prim_schwarz_run(const Pairs& P, const Shells& S, const int* list, int n, const double* boys, double* pp,
+                             float* qp, float* qg, cudaStream_t st)
+{
+    if (n > 0)
+        prim_schwarz_kernel<C><<<(n + PSW_PAIRS - 1) / PSW_PAIRS, 64, 0, st>>>(P, S, list, n, boys, pp, qp, qg);
 }
 
 }  // namespace pimd
