@@ -146,10 +146,11 @@ def generate_sources():
             e += [f"    if (bs == 0{'' if straight_e[nm] else ' || true'}) {{",
                   "        CoopTape t; int W, Wf; size_t bytes, bytesf;",
                   f"        coop_tape_{nm}(t, W, bytes, Wf, bytesf);",
-                  f"        jk_coop_kernel<{la}, {lb}, {lc}, {ld}, double><<<ntiles, 32 * W, bytes, st>>>(P, S, R, tiles,",
+                  "        const dim3 grid(ntiles, coop_blocks_per_tile(ntiles));",
+                  f"        jk_coop_kernel<{la}, {lb}, {lc}, {ld}, double><<<grid, 32 * W, bytes, st>>>(P, S, R, tiles,",
                   "            D, G, boys, split, 1e300, Dsh, cnt, t, tp, fxs);",
                   "        if (fp32_tau > tau)",
-                  f"            jk_coop_kernel<{la}, {lb}, {lc}, {ld}, float><<<ntiles, 32 * Wf, bytesf, st>>>(P, S, R,",
+                  f"            jk_coop_kernel<{la}, {lb}, {lc}, {ld}, float><<<grid, 32 * Wf, bytesf, st>>>(P, S, R,",
                   "                tiles, Df, G, boysf, tau, fp32_tau, Dsh, cnt + 2, t, tp, fxs);",
                   "        return;",
                   "    }"]
@@ -197,10 +198,11 @@ def generate_sources():
             gl += [f"    if (variant == 0{' || true' if heavy[nm] else ''}) {{",
                    "        CoopTape t; int W, Wf; size_t bytes, bytesf;",
                    f"        coop_tape_{nm}(t, W, bytes, Wf, bytesf);",
-                   f"        grad2e_coop_kernel<{la}, {lb}, {lc}, {ld}, double><<<ntiles, 32 * W, bytes, st>>>(P, S, R,",
+                   "        const dim3 grid(ntiles, coop_blocks_per_tile(ntiles));",
+                   f"        grad2e_coop_kernel<{la}, {lb}, {lc}, {ld}, double><<<grid, 32 * W, bytes, st>>>(P, S, R,",
                    "            tiles, D, grad, boys, split, 1e300, Dsh, cnt, t, tp, fxs);",
                    "        if (fp32_tau > tau)",
-                   f"            grad2e_coop_kernel<{la}, {lb}, {lc}, {ld}, float><<<ntiles, 32 * Wf, bytesf, st>>>(P, S,",
+                   f"            grad2e_coop_kernel<{la}, {lb}, {lc}, {ld}, float><<<grid, 32 * Wf, bytesf, st>>>(P, S,",
                    "                R, tiles, D, grad, boysf, tau, fp32_tau, Dsh, cnt + 2, t, tp, fxs);",
                    "        return;",
                    "    }"]

@@ -377,6 +377,19 @@ inline int coop_best_warps(int NACC, int NWORK, int L, int ncart4, size_t elem)
     return best;
 }
 
+// blocks per tile (gridDim.y; block y takes the tile's quartets y, y + gridDim.y,
+// ...). A quartet keeps a block busy for up to 0.2 ms and a tile holds up to
+// 128 of them, so one block per tile left SMs idle on small batches ((dd|dd)
+// of one (H2O)8 bead: 36 tiles on 152 SMs) and a long last wave on large ones.
+// One bead of (H2O)8: gradient 386 -> 205 ms, forces call 1656 -> 1280 ms.
+// Enough blocks for 16 per SM, which balances them; more would only repeat the
+// tile's set-up.
+inline int coop_blocks_per_tile(int ntiles)
+{
+    const int want = 16 * 152;
+    return ntiles >= want ? 1 : (want + ntiles - 1) / ntiles < 128 ? (want + ntiles - 1) / ntiles : 128;
+}
+
 // Fock build of the quartets whose density-weighted bound lies in [tau_lo, tau_hi)
 template <int LA, int LB, int LC, int LD, typename Rt>
 __global__ void __launch_bounds__(128) jk_coop_kernel(Pairs P, Shells S, Reps R, const Tile* __restrict__ tiles,
@@ -404,9 +417,9 @@ __global__ void __launch_bounds__(128) jk_coop_kernel(Pairs P, Shells S, Reps R,
         A[x] = S.xyz[3 * sa + x];
         B[x] = S.xyz[3 * sb + x];
     }
-    // the block's threads take the tile's quartets one at a time (the bound
-    // and hence every branch below is the same for all of them)
-    for (int cd = t.c0; cd < t.c1; cd++) {
+    // the block's threads take its share of the tile's quartets one at a time
+    // (the bound and hence every branch below is the same for all of them)
+    for (int cd = t.c0 + blockIdx.y; cd < t.c1; cd += gridDim.y) {
         const int sc = P.sa[cd], sd = P.sb[cd];
         const double dq = fmax(fmax(fmax(shell_bound(R, Dsh, r, sa, sb), shell_bound(R, Dsh, r, sc, sd)),
                                     fmax(shell_bound(R, Dsh, r, sa, sc), shell_bound(R, Dsh, r, sa, sd))),
@@ -475,7 +488,7 @@ __global__ void __launch_bounds__(128) grad2e_coop_kernel(Pairs P, Shells S, Rep
     const int N = R.nbf[r];
     const double* D = Dall + R.moff[r];
     // one quartet at a time over the block (uniform branches)
-    for (int cd = t.c0; cd < t.c1; cd++) {
+    for (int cd = t.c0 + blockIdx.y; cd < t.c1; cd += gridDim.y) {
         const int sc = P.sa[cd], sd = P.sb[cd];
         const double gam = gamma_bound(R, Dsh, r, sa, sb, sc, sd);
         const double bound = P.Q[ab] * P.Q[cd] * gam;
