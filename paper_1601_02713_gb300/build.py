@@ -343,7 +343,8 @@ def build(force: bool = False, jobs: int | None = None, verbose: bool = False) -
     work = []
     for f in HAND_WRITTEN:
         src = os.path.join(CSRC, f)
-        work.append((src, os.path.join(OBJ, f + ".o"), _deps_hash(src, common)))
+        deps = common + [os.path.join(GEN, "nuclear.cuh")] if f == "onee.cu" else common
+        work.append((src, os.path.join(OBJ, f + ".o"), _deps_hash(src, deps)))
     for src in tus:
         base = os.path.basename(src)
         deps = list(common)

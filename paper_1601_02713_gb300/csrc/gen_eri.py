@@ -738,11 +738,80 @@ def write_if_changed(path, text):
     return True
 
 
+# ---------------------------------------------------------------------------
+# nuclear attraction: straight-line V^m(a, b) recursion of one primitive pair
+# and one nucleus (onee.cu has the rule)
+# ---------------------------------------------------------------------------
+class NucGen:
+    def __init__(self):
+        self.memo = {}
+        self.lines = []
+
+    def get(self, e, f, m):
+        key = (e, f, m)
+        if key in self.memo:
+            return self.memo[key]
+        if sum(e) == 0 and sum(f) == 0:
+            self.memo[key] = f"F[{m}]"
+            return self.memo[key]
+        bra = sum(f) == 0
+        i = pick_dir(e if bra else f)
+        e1, f1 = (sub(e, i), f) if bra else (e, sub(f, i))
+        terms = [f"{'PA' if bra else 'PB'}[{i}] * {self.get(e1, f1, m)}", f"-PC[{i}] * {self.get(e1, f1, m + 1)}"]
+        for k, (e2, f2) in ((e1[i], (sub(e1, i), f1)), (f1[i], (e1, sub(f1, i)))):
+            if k > 0:
+                c = "o2p" if k == 1 else f"{k}.0 * o2p"
+                terms.append(f"{c} * ({self.get(e2, f2, m)} - {self.get(e2, f2, m + 1)})")
+        name = f"n{len(self.lines)}"
+        self.lines.append(f"const double {name} = {' + '.join(terms)};")
+        self.memo[key] = name
+        return name
+
+
+def gen_nuclear(la, lb):
+    """Two device functions of the shell pair (la, lb): nuc_<la><lb> adds the
+    attraction integrals (a|b) to out, nuc_grad_<la><lb> adds
+    sum_ab Dc_ab (2 alpha V(a + 1_x, b) - a_x V(a - 1_x, b)) to s[x]."""
+    arg = ("const double* F, const double PA[3], const double PB[3], const double PC[3], double o2p")
+    g = NucGen()
+    outs = [f"out[{k}] += {g.get(a, b, 0)};" for k, (a, b) in enumerate((a, b) for a in carts(la) for b in carts(lb))]
+    code = [f"static __device__ __forceinline__ void nuc_{la}{lb}({arg}, double* out)\n{{"]
+    code += ["    " + x for x in g.lines + outs] + ["}"]
+    g = NucGen()
+    outs = []
+    for k, (a, b) in enumerate((a, b) for a in carts(la) for b in carts(lb)):
+        for x in range(3):
+            v = f"ta * {g.get(add(a, x), b, 0)}"
+            if a[x] > 0:
+                v += f" - {a[x]}.0 * {g.get(sub(a, x), b, 0)}"
+            outs.append(f"s[{x}] = fma(Dc[{k}], {v}, s[{x}]);")
+    code += [f"static __device__ __forceinline__ void nuc_grad_{la}{lb}({arg}, double ta, const double* Dc, double* s)",
+             "{"]
+    code += ["    " + x for x in g.lines + outs] + ["}"]
+    return "\n".join(code) + "\n"
+
+
+def generate_nuclear(outdir):
+    import os
+    pairs = [(la, lb) for la in range(LMAX + 1) for lb in range(LMAX + 1)]
+    text = ["// Generated by gen_eri.py: nuclear attraction recursions of every shell pair.\n#pragma once\n\n"]
+    text += [gen_nuclear(la, lb) for la, lb in pairs]
+    for fn, tail in (("nuc", "double* out"), ("nuc_grad", "double ta, const double* Dc, double* s")):
+        names = ", ".join(t.split()[-1].lstrip("*") for t in tail.split(","))
+        text.append(f"template <int LA, int LB>\nstatic __device__ __forceinline__ void {fn}_of(const double* F, "
+                    f"const double PA[3], const double PB[3], const double PC[3], double o2p, {tail})\n{{\n")
+        for la, lb in pairs:
+            text.append(f"    if constexpr (LA == {la} && LB == {lb}) {fn}_{la}{lb}(F, PA, PB, PC, o2p, {names});\n")
+        text.append("}\n")
+    write_if_changed(os.path.join(outdir, "nuclear.cuh"), "".join(text))
+
+
 def generate(outdir):
     """Write one header per class (energy VRR/HRR, gradient VRR/HRR or tape).
     Returns per-class statistics."""
     import os
     os.makedirs(outdir, exist_ok=True)
+    generate_nuclear(outdir)
     stats = []
     for c in classes():
         la, lb, lc, ld = c

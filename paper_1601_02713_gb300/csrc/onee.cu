@@ -14,25 +14,15 @@
 //   V^m(0,0) = (2 pi / p) K F_m(p |PC|^2)     (and the same rule for b+1_i with PB).
 #include <math.h>
 
-#include "boys.cuh"
+#include "eri_kernels.cuh"
 #include "internal.h"
+#include "nuclear.cuh"
 
 namespace pimd {
 
 namespace {
 
 constexpr double kPi = 3.14159265358979323846;
-constexpr int NA1 = 20;   // Cartesian components of levels 0..3
-constexpr int NB1 = 10;   // levels 0..2
-constexpr int NM1 = 6;
-
-__device__ __forceinline__ int loff(int l) { return l * (l + 1) * (l + 2) / 6; }
-__device__ __forceinline__ int gidx(int x, int y, int z)
-{
-    const int l = x + y + z;
-    return loff(l) + (l - x) * (l - x + 1) / 2 + z;
-}
-
 __device__ __forceinline__ int cidx_host_dev(const int* e)
 {
     const int l = e[0] + e[1] + e[2];
@@ -52,78 +42,6 @@ __device__ __forceinline__ void cart_of_d(int l, int idx, int* e)
             }
             n++;
         }
-}
-
-__device__ __forceinline__ int dir_of(const int* e)
-{
-    return (e[0] >= e[1] && e[0] >= e[2]) ? 0 : (e[1] >= e[2] ? 1 : 2);
-}
-
-// V^m(a, b) tables for a levels 0..la, b levels 0..lb (m = 0 of levels la, lb
-// are the attraction integrals). Vt[(m * NA1 + ia) * NB1 + ib].
-__device__ void os_nuclear(int la, int lb, double p, const double* PA, const double* PB, const double* PC,
-                           const double* F, double pref, double* Vt)
-{
-    const int Lt = la + lb;
-    const double o2p = 0.5 / p;
-    for (int m = 0; m <= Lt; m++) Vt[(m * NA1 + 0) * NB1 + 0] = pref * F[m];
-    for (int l = 1; l <= la; l++) {
-        for (int c = 0; c < (l + 1) * (l + 2) / 2; c++) {
-            int e[3];
-            cart_of_d(l, c, e);
-            const int i = dir_of(e);
-            int e1[3] = {e[0], e[1], e[2]};
-            e1[i]--;
-            const int ia = gidx(e[0], e[1], e[2]), i1 = gidx(e1[0], e1[1], e1[2]);
-            int i2 = -1;
-            if (e1[i] > 0) {
-                int e2[3] = {e1[0], e1[1], e1[2]};
-                e2[i]--;
-                i2 = gidx(e2[0], e2[1], e2[2]);
-            }
-            for (int m = 0; m <= Lt - l; m++) {
-                double v = PA[i] * Vt[(m * NA1 + i1) * NB1] - PC[i] * Vt[((m + 1) * NA1 + i1) * NB1];
-                if (i2 >= 0) v += e1[i] * o2p * (Vt[(m * NA1 + i2) * NB1] - Vt[((m + 1) * NA1 + i2) * NB1]);
-                Vt[(m * NA1 + ia) * NB1] = v;
-            }
-        }
-    }
-    for (int lbb = 1; lbb <= lb; lbb++) {
-        for (int cb = 0; cb < (lbb + 1) * (lbb + 2) / 2; cb++) {
-            int f[3];
-            cart_of_d(lbb, cb, f);
-            const int i = dir_of(f);
-            int f1[3] = {f[0], f[1], f[2]};
-            f1[i]--;
-            const int ib = gidx(f[0], f[1], f[2]), j1 = gidx(f1[0], f1[1], f1[2]);
-            int j2 = -1;
-            if (f1[i] > 0) {
-                int f2[3] = {f1[0], f1[1], f1[2]};
-                f2[i]--;
-                j2 = gidx(f2[0], f2[1], f2[2]);
-            }
-            for (int l = 0; l <= la; l++)
-                for (int c = 0; c < (l + 1) * (l + 2) / 2; c++) {
-                    int e[3];
-                    cart_of_d(l, c, e);
-                    const int ia = gidx(e[0], e[1], e[2]);
-                    int ia1 = -1;
-                    if (e[i] > 0) {
-                        int e1[3] = {e[0], e[1], e[2]};
-                        e1[i]--;
-                        ia1 = gidx(e1[0], e1[1], e1[2]);
-                    }
-                    for (int m = 0; m <= Lt - l - lbb; m++) {
-                        double v = PB[i] * Vt[(m * NA1 + ia) * NB1 + j1] - PC[i] * Vt[((m + 1) * NA1 + ia) * NB1 + j1];
-                        if (ia1 >= 0)
-                            v += e[i] * o2p * (Vt[(m * NA1 + ia1) * NB1 + j1] - Vt[((m + 1) * NA1 + ia1) * NB1 + j1]);
-                        if (j2 >= 0)
-                            v += f1[i] * o2p * (Vt[(m * NA1 + ia) * NB1 + j2] - Vt[((m + 1) * NA1 + ia) * NB1 + j2]);
-                        Vt[(m * NA1 + ia) * NB1 + ib] = v;
-                    }
-                }
-        }
-    }
 }
 
 // 1-D overlap table S[i][j], i <= imax, j <= jmax (without the (pi/p)^{1/2} K factor)
@@ -156,77 +74,21 @@ __device__ __forceinline__ double kin_1d(const double S[6][5], int i, int j, dou
     return 0.5 * t;
 }
 
-// 2-index Cartesian -> spherical transform of block[na_c][nb_c] in place
-__device__ void sph2(int la, int lb, double* blk)
+// run(LA, LB) as compile-time constants for shells of angular momenta la, lb
+template <class F>
+__device__ __forceinline__ void by_l(int la, int lb, F&& run)
 {
-    const double s3 = 1.7320508075688772935;
-    const int nac = (la + 1) * (la + 2) / 2, nbc = (lb + 1) * (lb + 2) / 2;
-    double tmp[36];
-    int nas = nac;
-    if (la == 2) {
-        for (int j = 0; j < nbc; j++) {
-            const double xx = blk[0 * nbc + j], xy = blk[1 * nbc + j], xz = blk[2 * nbc + j], yy = blk[3 * nbc + j],
-                         yz = blk[4 * nbc + j], zz = blk[5 * nbc + j];
-            tmp[0 * nbc + j] = s3 * xy;
-            tmp[1 * nbc + j] = s3 * yz;
-            tmp[2 * nbc + j] = zz - 0.5 * (xx + yy);
-            tmp[3 * nbc + j] = s3 * xz;
-            tmp[4 * nbc + j] = 0.5 * s3 * (xx - yy);
-        }
-        nas = 5;
-        for (int k = 0; k < nas * nbc; k++) blk[k] = tmp[k];
-    }
-    if (lb == 2) {
-        for (int i = 0; i < nas; i++) {
-            const double* r = blk + i * 6;
-            const double xx = r[0], xy = r[1], xz = r[2], yy = r[3], yz = r[4], zz = r[5];
-            tmp[i * 5 + 0] = s3 * xy;
-            tmp[i * 5 + 1] = s3 * yz;
-            tmp[i * 5 + 2] = zz - 0.5 * (xx + yy);
-            tmp[i * 5 + 3] = s3 * xz;
-            tmp[i * 5 + 4] = 0.5 * s3 * (xx - yy);
-        }
-        for (int k = 0; k < nas * 5; k++) blk[k] = tmp[k];
-    }
-}
-
-// spherical block [na_s][nb_s] -> Cartesian-component weights [na_c][nb_c]
-// (transpose transform: sum_sph X_s I_s = sum_cart X_c I_c)
-__device__ void sph2_t(int la, int lb, const double* in, double* out)
-{
-    const double s3 = 1.7320508075688772935;
-    const int nac = (la + 1) * (la + 2) / 2, nbc = (lb + 1) * (lb + 2) / 2;
-    const int nas = la == 2 ? 5 : nac, nbs = lb == 2 ? 5 : nbc;
-    double tmp[36];
-    // first index
-    for (int j = 0; j < nbs; j++) {
-        if (la == 2) {
-            const double m2 = in[0 * nbs + j], m1 = in[1 * nbs + j], m0 = in[2 * nbs + j], p1 = in[3 * nbs + j],
-                         p2 = in[4 * nbs + j];
-            tmp[0 * nbs + j] = -0.5 * m0 + 0.5 * s3 * p2;
-            tmp[1 * nbs + j] = s3 * m2;
-            tmp[2 * nbs + j] = s3 * p1;
-            tmp[3 * nbs + j] = -0.5 * m0 - 0.5 * s3 * p2;
-            tmp[4 * nbs + j] = s3 * m1;
-            tmp[5 * nbs + j] = m0;
-        } else {
-            for (int i = 0; i < nac; i++) tmp[i * nbs + j] = in[i * nbs + j];
-        }
-    }
-    for (int i = 0; i < nac; i++) {
-        if (lb == 2) {
-            const double* r = tmp + i * 5;
-            const double m2 = r[0], m1 = r[1], m0 = r[2], p1 = r[3], p2 = r[4];
-            double* o = out + i * 6;
-            o[0] = -0.5 * m0 + 0.5 * s3 * p2;
-            o[1] = s3 * m2;
-            o[2] = s3 * p1;
-            o[3] = -0.5 * m0 - 0.5 * s3 * p2;
-            o[4] = s3 * m1;
-            o[5] = m0;
-        } else {
-            for (int j = 0; j < nbc; j++) out[i * nbc + j] = tmp[i * nbc + j];
-        }
+    using std::integral_constant;
+    switch (3 * la + lb) {
+    case 0: run(integral_constant<int, 0>(), integral_constant<int, 0>()); break;
+    case 1: run(integral_constant<int, 0>(), integral_constant<int, 1>()); break;
+    case 2: run(integral_constant<int, 0>(), integral_constant<int, 2>()); break;
+    case 3: run(integral_constant<int, 1>(), integral_constant<int, 0>()); break;
+    case 4: run(integral_constant<int, 1>(), integral_constant<int, 1>()); break;
+    case 5: run(integral_constant<int, 1>(), integral_constant<int, 2>()); break;
+    case 6: run(integral_constant<int, 2>(), integral_constant<int, 0>()); break;
+    case 7: run(integral_constant<int, 2>(), integral_constant<int, 1>()); break;
+    case 8: run(integral_constant<int, 2>(), integral_constant<int, 2>()); break;
     }
 }
 
@@ -269,317 +131,243 @@ __global__ void pair_data_kernel(Pairs P, int* npp, double* pp, Shells S, BasisP
     npp[g] = k;
 }
 
-// Cartesian S, T, V blocks of bra shell a (raised by dla with weight 2 alpha if
-// wa) and ket shell b, contracted. The nuclear attraction is summed over the
-// nuclei [c0, c1) unless single >= 0 (then only nucleus `single`).
-__device__ void one_e_blocks(int sa, int sb, int la, int lb, const Shells& S, const BasisPrimDev& B,
-                             const AtomsDev& At, int c0, int c1, const double* boys, double* Sb, double* Tb,
-                             double* Vb, bool want_st)
+__device__ __forceinline__ double lane_sum(double v)
 {
-    const int nac = (la + 1) * (la + 2) / 2, nbc = (lb + 1) * (lb + 2) / 2;
-    for (int k = 0; k < nac * nbc; k++) {
-        if (want_st) {
-            Sb[k] = 0.0;
-            Tb[k] = 0.0;
-        }
-        Vb[k] = 0.0;
-    }
-    double A[3], Bc[3], AB2 = 0.0;
-    for (int x = 0; x < 3; x++) {
-        A[x] = S.xyz[3 * sa + x];
-        Bc[x] = S.xyz[3 * sb + x];
-        AB2 += (A[x] - Bc[x]) * (A[x] - Bc[x]);
-    }
-    const int pa = B.sprim[sa], pb = B.sprim[sb];
-    for (int i = 0; i < B.snprim[sa]; i++)
-        for (int j = 0; j < B.snprim[sb]; j++) {
-            const double a = B.exps[pa + i], b = B.exps[pb + j];
-            const double p = a + b;
-            const double K = B.coefs[pa + i] * B.coefs[pb + j] * exp(-a * b / p * AB2);
-            double P[3], PA[3], PB[3];
-            for (int x = 0; x < 3; x++) {
-                P[x] = (a * A[x] + b * Bc[x]) / p;
-                PA[x] = P[x] - A[x];
-                PB[x] = P[x] - Bc[x];
-            }
-            if (want_st) {
-                double S1[3][6][5];
-                for (int x = 0; x < 3; x++) os_overlap_1d(la + 1, lb + 1, PA[x], PB[x], p, S1[x]);
-                const double pre = K * pow(kPi / p, 1.5);
-                for (int ia = 0; ia < nac; ia++) {
-                    int e[3];
-                    cart_of_d(la, ia, e);
-                    for (int ib = 0; ib < nbc; ib++) {
-                        int f[3];
-                        cart_of_d(lb, ib, f);
-                        const double sx = S1[0][e[0]][f[0]], sy = S1[1][e[1]][f[1]], sz = S1[2][e[2]][f[2]];
-                        const double tx = kin_1d(S1[0], e[0], f[0], a, b), ty = kin_1d(S1[1], e[1], f[1], a, b),
-                                     tz = kin_1d(S1[2], e[2], f[2], a, b);
-                        Sb[ia * nbc + ib] += pre * sx * sy * sz;
-                        Tb[ia * nbc + ib] += pre * (tx * sy * sz + sx * ty * sz + sx * sy * tz);
-                    }
-                }
-            }
-            double Vt[NM1 * NA1 * NB1];
-            for (int c = c0; c < c1; c++) {
-                double PC[3], PC2 = 0.0;
-                for (int x = 0; x < 3; x++) {
-                    PC[x] = P[x] - At.xyz[3 * c + x];
-                    PC2 += PC[x] * PC[x];
-                }
-                double F[NM1];
-                boys_eval_n(la + lb, p * PC2, boys, 1.0, F);
-                os_nuclear(la, lb, p, PA, PB, PC, F, -At.Z[c] * 2.0 * kPi / p * K, Vt);
-                for (int ia = 0; ia < nac; ia++) {
-                    int e[3];
-                    cart_of_d(la, ia, e);
-                    const int ga = gidx(e[0], e[1], e[2]);
-                    for (int ib = 0; ib < nbc; ib++) {
-                        int f[3];
-                        cart_of_d(lb, ib, f);
-                        Vb[ia * nbc + ib] += Vt[(0 * NA1 + ga) * NB1 + gidx(f[0], f[1], f[2])];
-                    }
-                }
-            }
-        }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
-__global__ void one_e_kernel(Pairs P, Shells S, BasisPrimDev B, AtomsDev At, Reps R, double* Sm, double* Tm,
-                             double* Vm, const double* boys)
+// primitive pair (i, j) of shells (sa, sb): exponents and Gaussian product
+struct PrimPair {
+    double a, b, p, K, P[3], PA[3], PB[3];
+    __device__ __forceinline__ PrimPair(const Shells& S, const BasisPrimDev& B, int sa, int sb, int i, int j)
+    {
+        const int pa = B.sprim[sa] + i, pb = B.sprim[sb] + j;
+        a = B.exps[pa];
+        b = B.exps[pb];
+        p = a + b;
+        double AB2 = 0.0;
+#pragma unroll
+        for (int x = 0; x < 3; x++) {
+            const double A = S.xyz[3 * sa + x], Bc = S.xyz[3 * sb + x];
+            AB2 += (A - Bc) * (A - Bc);
+            P[x] = (a * A + b * Bc) / p;
+            PA[x] = P[x] - A;
+            PB[x] = P[x] - Bc;
+        }
+        K = B.coefs[pa] * B.coefs[pb] * exp(-a * b / p * AB2);
+    }
+};
+
+// F[m] = -Z_c (2 pi / p) K F_m(p |P - C|^2) of nucleus c, m = 0..L; PC = P - C
+template <int L>
+__device__ __forceinline__ void nuclear_boys(const PrimPair& g, const AtomsDev& At, int c, const double* boys,
+                                             double PC[3], double* F)
 {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= P.n) return;
-    const int sa = P.sa[g], sb = P.sb[g];
-    const int la = S.l[sa], lb = S.l[sb];
-    const int r = S.rep[sa];
-    double Sb[36], Tb[36], Vb[36];
-    one_e_blocks(sa, sb, la, lb, S, B, At, At.rep_atom0[r], At.rep_atom0[r + 1], boys, Sb, Tb, Vb, true);
-    sph2(la, lb, Sb);
-    sph2(la, lb, Tb);
-    sph2(la, lb, Vb);
-    const int na = nsph(la), nb = nsph(lb);
+    double r2 = 0.0;
+#pragma unroll
+    for (int x = 0; x < 3; x++) {
+        PC[x] = g.P[x] - At.xyz[3 * c + x];
+        r2 += PC[x] * PC[x];
+    }
+    boys_eval<L>(g.p * r2, boys, -At.Z[c] * 2.0 * kPi / g.p * g.K, F);
+}
+
+// S, T, V of one shell pair by one warp. The nuclear attraction is the work:
+// (primitive pair, nucleus) is one lane's unit, 9 x 24 of them for (H2O)8, and
+// its recursion straight-line code; the lanes' Cartesian blocks are summed over
+// the warp. Bound by the latency of a lane's FP64 chain: one thread per pair
+// with the recursion's tables in local memory, as before, took 12.8 ms for one
+// bead of (H2O)8.
+template <int LA, int LB>
+__device__ __forceinline__ void one_e_pair(int g, const Pairs& P, const Shells& S, const BasisPrimDev& B,
+                                           const AtomsDev& At, const Reps& R, double* Sm, double* Tm, double* Vm,
+                                           const double* boys)
+{
+    constexpr int nac = ncart(LA), nbc = ncart(LB), n = nac * nbc;
+    const int sa = P.sa[g], sb = P.sb[g], r = S.rep[sa], lane = threadIdx.x & 31;
+    const int na = B.snprim[sa], np = na * B.snprim[sb];
+    const int c0 = At.rep_atom0[r], nc = At.rep_atom0[r + 1] - c0;
+    double Sb[n], Tb[n], Vb[n];
+#pragma unroll
+    for (int k = 0; k < n; k++) Sb[k] = Tb[k] = Vb[k] = 0.0;
+    for (int u = lane; u < np * nc; u += 32) {
+        const PrimPair q(S, B, sa, sb, (u % np) % na, (u % np) / na);
+        double PC[3], F[LA + LB + 1];
+        nuclear_boys<LA + LB>(q, At, c0 + u / np, boys, PC, F);
+        nuc_of<LA, LB>(F, q.PA, q.PB, PC, 0.5 / q.p, Vb);
+    }
+    if (lane < np) {
+        const PrimPair q(S, B, sa, sb, lane % na, lane / na);
+        double S1[3][6][5];
+        for (int x = 0; x < 3; x++) os_overlap_1d(LA + 1, LB + 1, q.PA[x], q.PB[x], q.p, S1[x]);
+        const double pre = q.K * pow(kPi / q.p, 1.5);
+        for (int ia = 0; ia < nac; ia++) {
+            int e[3];
+            cart_of_d(LA, ia, e);
+            for (int ib = 0; ib < nbc; ib++) {
+                int f[3];
+                cart_of_d(LB, ib, f);
+                const double sx = S1[0][e[0]][f[0]], sy = S1[1][e[1]][f[1]], sz = S1[2][e[2]][f[2]];
+                const double tx = kin_1d(S1[0], e[0], f[0], q.a, q.b), ty = kin_1d(S1[1], e[1], f[1], q.a, q.b),
+                             tz = kin_1d(S1[2], e[2], f[2], q.a, q.b);
+                Sb[ia * nbc + ib] = pre * sx * sy * sz;
+                Tb[ia * nbc + ib] = pre * (tx * sy * sz + sx * ty * sz + sx * sy * tz);
+            }
+        }
+    }
     const int N = R.nbf[r];
     const size_t off = R.moff[r];
     const int fa = S.bf[sa], fb = S.bf[sb];
-    for (int i = 0; i < na; i++)
-        for (int j = 0; j < nb; j++) {
-            const size_t u = off + (size_t)(fa + i) * N + fb + j, v = off + (size_t)(fb + j) * N + fa + i;
-            Sm[u] = Sb[i * nb + j];
-            Sm[v] = Sb[i * nb + j];
-            Tm[u] = Tb[i * nb + j];
-            Tm[v] = Tb[i * nb + j];
-            Vm[u] = Vb[i * nb + j];
-            Vm[v] = Vb[i * nb + j];
-        }
+    double* const out[3] = {Sm, Tm, Vm};
+    double* const in[3] = {Sb, Tb, Vb};
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        double c[n], t[n];
+#pragma unroll
+        for (int e = 0; e < n; e++) c[e] = lane_sum(in[k][e]);
+        sph_index<1, LA, nbc>(c, t);
+        sph_index<nsph(LA), LB, 1>(t, c);
+        if (lane == 0)
+#pragma unroll
+            for (int i = 0; i < nsph(LA); i++)
+#pragma unroll
+                for (int j = 0; j < nsph(LB); j++) {
+                    out[k][off + (size_t)(fa + i) * N + fb + j] = c[i * nsph(LB) + j];
+                    out[k][off + (size_t)(fb + j) * N + fa + i] = c[i * nsph(LB) + j];
+                }
+    }
 }
 
-// derivative of the bra Gaussian: d/dA_x g_a = 2 alpha g_{a+1_x} - a_x g_{a-1_x}
-// One thread per (pair, orientation).
-__global__ void grad_1e_kernel(Pairs P, Shells S, BasisPrimDev B, AtomsDev At, Reps R, const double* D,
-                               const double* W, double* grad, const double* boys, double fxs)
+// one warp per pair
+__global__ void __launch_bounds__(64) one_e_kernel(Pairs P, Shells S, BasisPrimDev B, AtomsDev At, Reps R, double* Sm,
+                                                   double* Tm, double* Vm, const double* boys)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (g >= P.n) return;
+    const int la = S.l[P.sa[g]], lb = S.l[P.sb[g]];
+    auto run = [&](auto a, auto b) {
+        one_e_pair<decltype(a)::value, decltype(b)::value>(g, P, S, B, At, R, Sm, Tm, Vm, boys);
+    };
+    by_l(la, lb, run);
+}
+
+// derivative of the bra Gaussian: d/dA_x g_a = 2 alpha g_{a+1_x} - a_x g_{a-1_x},
+// of one (pair, orientation) by one warp. Every term is contracted with the
+// density as soon as it is made, so a lane keeps three sums instead of
+// derivative blocks. Nuclear attraction: the lanes take the nuclei, G lanes to
+// a nucleus (its primitive pairs split over them) where there are fewer than
+// 32; one bead of (H2O)8 with a thread per (pair, orientation): 62.7 ms.
+template <int LA, int LB>
+__device__ __forceinline__ void grad_1e_pair(int sa, int sb, const Shells& S, const BasisPrimDev& B,
+                                             const AtomsDev& At, const Reps& R, const double* D, const double* W,
+                                             double* grad, const double* boys, double fxs)
+{
+    constexpr int nac = ncart(LA), nbc = ncart(LB), nas = nsph(LA), nbs = nsph(LB);
+    const int r = S.rep[sa], N = R.nbf[r], lane = threadIdx.x & 31;
+    const size_t off = R.moff[r] + (size_t)S.bf[sa] * N + S.bf[sb];
+    const int na = B.snprim[sa], np = na * B.snprim[sb];
+    // density block in Cartesian-component form (sum_sph X_s I_s = sum_cart X_c I_c)
+    auto load = [&](const double* M, double* c) {
+        double t[nac * nbc];
+#pragma unroll
+        for (int i = 0; i < nas; i++)
+#pragma unroll
+            for (int j = 0; j < nbs; j++) c[i * nbs + j] = __ldg(M + off + (size_t)i * N + j);
+        sph_index_t<1, LA, nbs>(c, t);
+        sph_index_t<nac, LB, 1>(t, c);
+    };
+    double Dc[nac * nbc];
+    load(D, Dc);
+    double ga[3] = {0.0, 0.0, 0.0};
+    // nuclear attraction: basis-function term on the bra atom and, by
+    // translational invariance of the three-centre integral (dA + dB + dC = 0,
+    // the ket term equal to the bra term by symmetry), the operator term
+    // -2 sum D dV^C/dA on nucleus C itself
+    const int c0 = At.rep_atom0[r], nc = At.rep_atom0[r + 1] - c0;
+    const int G = nc >= 32 ? 1 : nc >= 16 ? 2 : nc >= 8 ? 4 : nc >= 4 ? 8 : 16;
+    for (int cb = 0; cb < nc; cb += 32 / G) {
+        const int c = cb + lane / G;
+        double s[3] = {0.0, 0.0, 0.0};
+        if (c < nc)
+            for (int k = lane % G; k < np; k += G) {
+                const PrimPair q(S, B, sa, sb, k % na, k / na);
+                double PC[3], F[LA + LB + 2];
+                nuclear_boys<LA + LB + 1>(q, At, c0 + c, boys, PC, F);
+                nuc_grad_of<LA, LB>(F, q.PA, q.PB, PC, 0.5 / q.p, 2.0 * q.a, Dc, s);
+            }
+#pragma unroll
+        for (int x = 0; x < 3; x++) {
+            s[x] *= 2.0;
+            for (int o = 1; o < G; o <<= 1) s[x] += __shfl_xor_sync(0xffffffffu, s[x], o);
+            if (c < nc && lane % G == 0) {
+                ga[x] += s[x];
+                det_add(grad + 3 * (c0 + c) + x, -s[x], fxs);
+            }
+        }
+    }
+    // overlap and kinetic energy: a lane per primitive pair
+    if (lane < np) {
+        double Wc[nac * nbc];
+        load(W, Wc);
+        const PrimPair q(S, B, sa, sb, lane % na, lane / na);
+        double S1[3][6][5];
+        for (int x = 0; x < 3; x++) os_overlap_1d(LA + 2, LB + 1, q.PA[x], q.PB[x], q.p, S1[x]);
+        const double pre = 2.0 * q.K * pow(kPi / q.p, 1.5);
+        // components of level LA + 1 with weight 2 alpha, of level LA - 1 with -a_x
+        for (int lev = 0; lev < (LA > 0 ? 2 : 1); lev++) {
+            const int lq = lev == 0 ? LA + 1 : LA - 1;
+            for (int iq = 0; iq < ncart(lq); iq++) {
+                int e[3];
+                cart_of_d(lq, iq, e);
+                for (int ib = 0; ib < nbc; ib++) {
+                    int f[3];
+                    cart_of_d(LB, ib, f);
+                    const double sx = S1[0][e[0]][f[0]], sy = S1[1][e[1]][f[1]], sz = S1[2][e[2]][f[2]];
+                    const double tx = kin_1d(S1[0], e[0], f[0], q.a, q.b), ty = kin_1d(S1[1], e[1], f[1], q.a, q.b),
+                                 tz = kin_1d(S1[2], e[2], f[2], q.a, q.b);
+                    const double sv = pre * sx * sy * sz;
+                    const double tv = pre * (tx * sy * sz + sx * ty * sz + sx * sy * tz);
+#pragma unroll
+                    for (int x = 0; x < 3; x++) {
+                        // the component this one is the x-derivative of
+                        int d[3] = {e[0], e[1], e[2]};
+                        d[x] += lev == 0 ? -1 : 1;
+                        if (d[x] < 0) continue;
+                        const int k = cidx_host_dev(d) * nbc + ib;
+                        ga[x] += (lev == 0 ? 2.0 * q.a : -(double)d[x]) * (Dc[k] * tv - Wc[k] * sv);
+                    }
+                }
+            }
+        }
+    }
+    const int atom_a = S.atom[sa];
+#pragma unroll
+    for (int x = 0; x < 3; x++) {
+        const double v = lane_sum(ga[x]);
+        if (lane == 0) det_add(grad + 3 * atom_a + x, v, fxs);
+    }
+}
+
+// one warp per (pair, orientation)
+__global__ void __launch_bounds__(64) grad_1e_kernel(Pairs P, Shells S, BasisPrimDev B, AtomsDev At, Reps R,
+                                                     const double* D, const double* W, double* grad,
+                                                     const double* boys, double fxs)
+{
+    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (t >= 2 * P.n) return;
-    const int g = t >> 1, orient = t & 1;
-    int sa = P.sa[g], sb = P.sb[g];
-    if (orient) {
+    int sa = P.sa[t >> 1], sb = P.sb[t >> 1];
+    if (t & 1) {
         if (sa == sb) return;
         const int tmp = sa;
         sa = sb;
         sb = tmp;
     }
-    const int la = S.l[sa], lb = S.l[sb];
-    const int r = S.rep[sa];
-    const int N = R.nbf[r];
-    const size_t off = R.moff[r];
-    const int fa = S.bf[sa], fb = S.bf[sb];
-    const int nas = nsph(la), nbs = nsph(lb);
-    const int nac = ncart(la), nbc = ncart(lb);
-    // density and energy-weighted density blocks in Cartesian-component form
-    double Ds[25], Ws[25], Dc[36], Wc[36];
-    for (int i = 0; i < nas; i++)
-        for (int j = 0; j < nbs; j++) {
-            Ds[i * nbs + j] = D[off + (size_t)(fa + i) * N + fb + j];
-            Ws[i * nbs + j] = W[off + (size_t)(fa + i) * N + fb + j];
-        }
-    sph2_t(la, lb, Ds, Dc);
-    sph2_t(la, lb, Ws, Wc);
-    const int c0 = At.rep_atom0[r], c1 = At.rep_atom0[r + 1];
-    const int atom_a = S.atom[sa];
-    double ga[3] = {0.0, 0.0, 0.0};
-    // raised and lowered bra blocks of one bra primitive (the weight 2 alpha
-    // is per primitive): S, T summed over nuclei, V per nucleus
-    double Su[60], Tu[60], Vu[60], Sd[18], Td[18], Vd[18];
-    const int pa = B.sprim[sa];
-    const int ncu = ncart(la + 1), ncd = la > 0 ? ncart(la - 1) : 0;
-    // S and T derivative parts
-    {
-        double dS[3][36], dT[3][36];
-        for (int x = 0; x < 3; x++)
-            for (int k = 0; k < nac * nbc; k++) dS[x][k] = dT[x][k] = 0.0;
-        for (int i = 0; i < B.snprim[sa]; i++) {
-            const double a = B.exps[pa + i];
-            // raised
-            {
-                double A[3], Bc[3], AB2 = 0.0;
-                for (int x = 0; x < 3; x++) {
-                    A[x] = S.xyz[3 * sa + x];
-                    Bc[x] = S.xyz[3 * sb + x];
-                    AB2 += (A[x] - Bc[x]) * (A[x] - Bc[x]);
-                }
-                const int pb = B.sprim[sb];
-                for (int k = 0; k < ncu * nbc; k++) Su[k] = Tu[k] = 0.0;
-                for (int k = 0; k < ncd * nbc; k++) Sd[k] = Td[k] = 0.0;
-                for (int j = 0; j < B.snprim[sb]; j++) {
-                    const double b = B.exps[pb + j];
-                    const double p = a + b;
-                    const double K = B.coefs[pa + i] * B.coefs[pb + j] * exp(-a * b / p * AB2);
-                    double PA[3], PB[3];
-                    for (int x = 0; x < 3; x++) {
-                        const double Px = (a * A[x] + b * Bc[x]) / p;
-                        PA[x] = Px - A[x];
-                        PB[x] = Px - Bc[x];
-                    }
-                    double S1[3][6][5];
-                    for (int x = 0; x < 3; x++) os_overlap_1d(la + 2, lb + 1, PA[x], PB[x], p, S1[x]);
-                    const double pre = K * pow(kPi / p, 1.5);
-                    for (int lev = 0; lev < 2; lev++) {
-                        const int lq = lev == 0 ? la + 1 : la - 1;
-                        if (lq < 0) continue;
-                        const int nq = ncart(lq);
-                        for (int ia = 0; ia < nq; ia++) {
-                            int e[3];
-                            cart_of_d(lq, ia, e);
-                            for (int ib = 0; ib < nbc; ib++) {
-                                int f[3];
-                                cart_of_d(lb, ib, f);
-                                const double sx = S1[0][e[0]][f[0]], sy = S1[1][e[1]][f[1]], sz = S1[2][e[2]][f[2]];
-                                const double tx = kin_1d(S1[0], e[0], f[0], a, b),
-                                             ty = kin_1d(S1[1], e[1], f[1], a, b),
-                                             tz = kin_1d(S1[2], e[2], f[2], a, b);
-                                const double s = pre * sx * sy * sz;
-                                const double tk = pre * (tx * sy * sz + sx * ty * sz + sx * sy * tz);
-                                if (lev == 0) {
-                                    Su[ia * nbc + ib] += s;
-                                    Tu[ia * nbc + ib] += tk;
-                                } else {
-                                    Sd[ia * nbc + ib] += s;
-                                    Td[ia * nbc + ib] += tk;
-                                }
-                            }
-                        }
-                    }
-                }
-                for (int ia = 0; ia < nac; ia++) {
-                    int e[3];
-                    cart_of_d(la, ia, e);
-                    for (int x = 0; x < 3; x++) {
-                        int eu[3] = {e[0], e[1], e[2]};
-                        eu[x]++;
-                        const int iu = cidx_host_dev(eu);
-                        for (int ib = 0; ib < nbc; ib++) {
-                            double vs = 2.0 * a * Su[iu * nbc + ib], vt = 2.0 * a * Tu[iu * nbc + ib];
-                            if (e[x] > 0) {
-                                int ed[3] = {e[0], e[1], e[2]};
-                                ed[x]--;
-                                const int id = cidx_host_dev(ed);
-                                vs -= e[x] * Sd[id * nbc + ib];
-                                vt -= e[x] * Td[id * nbc + ib];
-                            }
-                            dS[x][ia * nbc + ib] += vs;
-                            dT[x][ia * nbc + ib] += vt;
-                        }
-                    }
-                }
-            }
-        }
-        for (int x = 0; x < 3; x++) {
-            double s = 0.0;
-            for (int k = 0; k < nac * nbc; k++) s += 2.0 * (Dc[k] * dT[x][k] - Wc[k] * dS[x][k]);
-            ga[x] += s;
-        }
-    }
-    // nuclear attraction, nucleus by nucleus: basis-function term on the bra
-    // atom and, by translational invariance of the three-centre integral
-    // (dA + dB + dC = 0, the ket term equal to the bra term by symmetry), the
-    // operator term -2 sum D dV^C/dA on nucleus C itself.
-    for (int c = c0; c < c1; c++) {
-        double dV[3][36];
-        for (int x = 0; x < 3; x++)
-            for (int k = 0; k < nac * nbc; k++) dV[x][k] = 0.0;
-        for (int i = 0; i < B.snprim[sa]; i++) {
-            const double a = B.exps[pa + i];
-            double A[3], Bc[3], AB2 = 0.0;
-            for (int x = 0; x < 3; x++) {
-                A[x] = S.xyz[3 * sa + x];
-                Bc[x] = S.xyz[3 * sb + x];
-                AB2 += (A[x] - Bc[x]) * (A[x] - Bc[x]);
-            }
-            const int pb = B.sprim[sb];
-            for (int k = 0; k < ncu * nbc; k++) Vu[k] = 0.0;
-            for (int k = 0; k < ncd * nbc; k++) Vd[k] = 0.0;
-            for (int j = 0; j < B.snprim[sb]; j++) {
-                const double b = B.exps[pb + j];
-                const double p = a + b;
-                const double K = B.coefs[pa + i] * B.coefs[pb + j] * exp(-a * b / p * AB2);
-                double PA[3], PB[3], PC[3], PC2 = 0.0;
-                for (int x = 0; x < 3; x++) {
-                    const double Px = (a * A[x] + b * Bc[x]) / p;
-                    PA[x] = Px - A[x];
-                    PB[x] = Px - Bc[x];
-                    PC[x] = Px - At.xyz[3 * c + x];
-                    PC2 += PC[x] * PC[x];
-                }
-                double F[NM1];
-                boys_eval_n(la + 1 + lb, p * PC2, boys, 1.0, F);
-                double Vt[NM1 * NA1 * NB1];
-                os_nuclear(la + 1, lb, p, PA, PB, PC, F, -At.Z[c] * 2.0 * kPi / p * K, Vt);
-                for (int lev = 0; lev < 2; lev++) {
-                    const int lq = lev == 0 ? la + 1 : la - 1;
-                    if (lq < 0) continue;
-                    for (int ia = 0; ia < ncart(lq); ia++) {
-                        int e[3];
-                        cart_of_d(lq, ia, e);
-                        const int gq = gidx(e[0], e[1], e[2]);
-                        for (int ib = 0; ib < nbc; ib++) {
-                            int f[3];
-                            cart_of_d(lb, ib, f);
-                            const double v = Vt[(0 * NA1 + gq) * NB1 + gidx(f[0], f[1], f[2])];
-                            if (lev == 0)
-                                Vu[ia * nbc + ib] += v;
-                            else
-                                Vd[ia * nbc + ib] += v;
-                        }
-                    }
-                }
-            }
-            for (int ia = 0; ia < nac; ia++) {
-                int e[3];
-                cart_of_d(la, ia, e);
-                for (int x = 0; x < 3; x++) {
-                    int eu[3] = {e[0], e[1], e[2]};
-                    eu[x]++;
-                    const int iu = cidx_host_dev(eu);
-                    for (int ib = 0; ib < nbc; ib++) {
-                        double v = 2.0 * a * Vu[iu * nbc + ib];
-                        if (e[x] > 0) {
-                            int ed[3] = {e[0], e[1], e[2]};
-                            ed[x]--;
-                            v -= e[x] * Vd[cidx_host_dev(ed) * nbc + ib];
-                        }
-                        dV[x][ia * nbc + ib] += v;
-                    }
-                }
-            }
-        }
-        for (int x = 0; x < 3; x++) {
-            double s = 0.0;
-            for (int k = 0; k < nac * nbc; k++) s += 2.0 * Dc[k] * dV[x][k];
-            ga[x] += s;
-            det_add(grad + 3 * c + x, -s, fxs);
-        }
-    }
-    for (int x = 0; x < 3; x++) det_add(grad + 3 * atom_a + x, ga[x], fxs);
+    auto run = [&](auto a, auto b) {
+        grad_1e_pair<decltype(a)::value, decltype(b)::value>(sa, sb, S, B, At, R, D, W, grad, boys, fxs);
+    };
+    by_l(S.l[sa], S.l[sb], run);
 }
 
 __global__ void vnn_kernel(AtomsDev At, int natom, const int* atom_rep, double* enn, double* grad, double fxs)
@@ -685,7 +473,7 @@ void launch_one_electron(const Pairs& P, const Shells& S, const BasisPrimDev& B,
                          const Reps& R, double* Sm, double* Tm, double* Vm, const double* boys, cudaStream_t st)
 {
     if (P.n == 0) return;
-    one_e_kernel<<<(P.n + 63) / 64, 64, 0, st>>>(P, S, B, At, R, Sm, Tm, Vm, boys);
+    one_e_kernel<<<(P.n + 1) / 2, 64, 0, st>>>(P, S, B, At, R, Sm, Tm, Vm, boys);
 }
 
 void launch_grad_1e(const Pairs& P, const Shells& S, const BasisPrimDev& B, const AtomsDev& At, const Reps& R,
@@ -693,7 +481,7 @@ void launch_grad_1e(const Pairs& P, const Shells& S, const BasisPrimDev& B, cons
                     cudaStream_t st)
 {
     if (P.n == 0) return;
-    grad_1e_kernel<<<(2 * P.n + 63) / 64, 64, 0, st>>>(P, S, B, At, R, D, W, grad, boys, fxs);
+    grad_1e_kernel<<<P.n, 64, 0, st>>>(P, S, B, At, R, D, W, grad, boys, fxs);
 }
 
 void launch_vnn(const AtomsDev& At, int natom_total, const int* atom_rep, double* enn, double* grad,
