@@ -121,6 +121,8 @@ def generate_sources():
     coop_e = {s[0]: s[7] for s in stats}
     coop_g = {s[0]: s[8] for s in stats}
     straight_e = {s[0]: s[9] for s in stats}
+    df_e = {s[0]: s[10] for s in stats}
+    df_g = {s[0]: s[11] for s in stats}
     classes = g.classes()
     names = [g.cls_name(c) for c in classes]
     tus = []
@@ -136,7 +138,7 @@ def generate_sources():
         # bs > 0: straight-line kernel with bs threads per block; bs == 0: the
         # cooperative tape kernel
         e += [f"void launch_jk_{nm}(const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles,",
-              "                     const double* D, const float* Df, double* G, const double* boys,",
+              "                     const double* D, const float* Df, const DfBuild& df, double* G, const double* boys,",
               "                     const float* boysf, double tau, double fp32_tau, const double* Dsh,",
               "                     unsigned long long* cnt, int bs, double tp, double fxs, cudaStream_t st)",
               "{",
@@ -144,6 +146,7 @@ def generate_sources():
               "    const double split = fp32_tau > tau ? fp32_tau : tau;"]
         if coop_e[nm]:
             e += [f"    if (bs == 0{'' if straight_e[nm] else ' || true'}) {{",
+                  "        if (df.stage == 1) return;",
                   "        CoopTape t; int W, Wf; size_t bytes, bytesf;",
                   f"        coop_tape_{nm}(t, W, bytes, Wf, bytesf);",
                   "        const dim3 grid(ntiles, coop_blocks_per_tile(ntiles));",
@@ -156,7 +159,16 @@ def generate_sources():
                   "    }"]
         if straight_e[nm]:
             e += ["    const int b = bs > 0 ? bs : 128;",
-                  f"    jk_kernel<Cls_{nm}, double><<<ntiles, b, 0, st>>>(P, S, R, tiles, D, G, boys, split, 1e300, Dsh, cnt,",
+                  "    const dim3 grid(ntiles, jk_blocks_per_tile(ntiles));"]
+            if df_e[nm]:
+                e += ["    const double top = df.tau > split ? df.tau : split;",
+                      "    if (top > split && df.stage != 2)",
+                      f"        jk_kernel<Cls_{nm}, dfloat><<<grid, b, 0, st>>>(P, S, R, tiles, df.D, G, df.boys, split, top,",
+                      "                                                        Dsh, cnt, tp, fxs);"]
+            else:
+                e += ["    const double top = split;"]
+            e += ["    if (df.stage == 1) return;",
+                  f"    jk_kernel<Cls_{nm}, double><<<grid, b, 0, st>>>(P, S, R, tiles, D, G, boys, top, 1e300, Dsh, cnt,",
                   "                                                      tp, fxs);",
                   "    if (fp32_tau > tau)",
                   f"        jk_kernel<Cls_{nm}, float><<<ntiles, b, 0, st>>>(P, S, R, tiles, Df, G, boysf, tau, fp32_tau, Dsh,",
@@ -188,7 +200,8 @@ def generate_sources():
             gl.append(f"void grad2e_upload_{nm}() {{}}")
         # variant 0: cooperative tape kernel, 1: straight-line kernel with bs threads
         gl += [f"void launch_grad2e_{nm}(const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles,",
-               "                        const double* D, double* grad, const double* boys, const float* boysf,",
+               "                        const double* D, const DfBuild& df, double* grad, const double* boys,",
+               "                        const float* boysf,",
                "                        double tau, double fp32_tau, const double* Dsh, unsigned long long* cnt,",
                "                        int variant, int bs, double tp, double fxs, cudaStream_t st)",
                "{",
@@ -196,6 +209,7 @@ def generate_sources():
                "    const double split = fp32_tau > tau ? fp32_tau : tau;"]
         if coop_g[nm]:
             gl += [f"    if (variant == 0{' || true' if heavy[nm] else ''}) {{",
+                   "        if (df.stage == 1) return;",
                    "        CoopTape t; int W, Wf; size_t bytes, bytesf;",
                    f"        coop_tape_{nm}(t, W, bytes, Wf, bytesf);",
                    "        const dim3 grid(ntiles, coop_blocks_per_tile(ntiles));",
@@ -208,7 +222,16 @@ def generate_sources():
                    "    }"]
         if not heavy[nm]:
             gl += ["    const int b = bs > 0 ? bs : 128;",
-                   f"    grad2e_kernel<GCls_{nm}, double><<<ntiles, b, 0, st>>>(P, S, R, tiles, D, grad, boys, split, 1e300, Dsh,",
+                   "    const dim3 grid(ntiles, jk_blocks_per_tile(ntiles));"]
+            if df_g[nm]:
+                gl += ["    const double top = df.tau > split ? df.tau : split;",
+                       "    if (top > split && df.stage != 2)",
+                       f"        grad2e_kernel<GCls_{nm}, dfloat><<<grid, b, 0, st>>>(P, S, R, tiles, df.D, grad, df.boys,",
+                       "                                                            split, top, Dsh, cnt, tp, fxs);"]
+            else:
+                gl += ["    const double top = split;"]
+            gl += ["    if (df.stage == 1) return;",
+                   f"    grad2e_kernel<GCls_{nm}, double><<<grid, b, 0, st>>>(P, S, R, tiles, D, grad, boys, top, 1e300, Dsh,",
                    "                                                            cnt, tp, fxs);",
                    "    if (fp32_tau > tau)",
                    f"        grad2e_kernel<GCls_{nm}, float><<<ntiles, b, 0, st>>>(P, S, R, tiles, D, grad, boysf, tau, fp32_tau,",
@@ -220,13 +243,13 @@ def generate_sources():
         tus.append(p)
     # dispatch
     d = ['#include "internal.h"', "namespace pimd {"]
-    sig_jk = ("const Pairs&, const Shells&, const Reps&, const Tile*, int, const double*, const float*, double*, "
-              "const double*, const float*, double, double, const double*, unsigned long long*, int, double, "
-              "double, cudaStream_t")
+    sig_jk = ("const Pairs&, const Shells&, const Reps&, const Tile*, int, const double*, const float*, "
+              "const DfBuild&, double*, const double*, const float*, double, double, const double*, "
+              "unsigned long long*, int, double, double, cudaStream_t")
     sig_sw = "const Pairs&, const Shells&, const int*, int, const double*, double*, cudaStream_t"
     sig_psw = "const Pairs&, const Shells&, const int*, int, const double*, double*, float*, float*, cudaStream_t"
-    sig_g = ("const Pairs&, const Shells&, const Reps&, const Tile*, int, const double*, double*, const double*, "
-             "const float*, double, double, const double*, unsigned long long*, int, int, double, double, cudaStream_t")
+    sig_g = ("const Pairs&, const Shells&, const Reps&, const Tile*, int, const double*, const DfBuild&, double*, "
+             "const double*, const float*, double, double, const double*, unsigned long long*, int, int, double, double, cudaStream_t")
     for c, nm in zip(classes, names):
         d.append(f"void launch_jk_{nm}({sig_jk});")
         if (c[0], c[1]) == (c[2], c[3]):
@@ -264,11 +287,11 @@ def generate_sources():
     d.append(f"typedef void (*JkFn)({sig_jk});")
     d.append("static const JkFn jk_tab[] = {" + ", ".join(f"launch_jk_{nm}" for nm in names) + "};")
     d.append("void launch_jk(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles, "
-             "const double* D, const float* Df, double* G, const double* boys, const float* boysf, double tau, "
-             "double fp32_tau, const double* Dsh, unsigned long long* cnt, int bs, double tau_prim, double fxs, "
-             "cudaStream_t st)")
-    d.append("{ jk_tab[cp](P, S, R, tiles, ntiles, D, Df, G, boys, boysf, tau, fp32_tau, Dsh, cnt, bs, tau_prim, fxs, st); }")
-    for fn, tab in (("class_pair_coop", coop_e), ("class_pair_straight", straight_e), ("grad_pair_coop", coop_g),
+             "const double* D, const float* Df, const DfBuild& df, double* G, const double* boys, const float* boysf, "
+             "double tau, double fp32_tau, const double* Dsh, unsigned long long* cnt, int bs, double tau_prim, "
+             "double fxs, cudaStream_t st)")
+    d.append("{ jk_tab[cp](P, S, R, tiles, ntiles, D, Df, df, G, boys, boysf, tau, fp32_tau, Dsh, cnt, bs, tau_prim, fxs, st); }")
+    for fn, tab in (("class_pair_coop", coop_e), ("class_pair_straight", straight_e), ("grad_pair_coop", coop_g), ("class_pair_df", df_e), ("grad_pair_df", df_g),
                     ("grad_pair_straight", {nm: not heavy[nm] for nm in names})):
         d.append(f"bool {fn}(int cp)")
         d.append("{")
@@ -290,10 +313,10 @@ def generate_sources():
     d.append("static const GFn g_tab[] = {" + ", ".join(f"launch_grad2e_{nm}" for nm in names) + "};")
 
     d.append("void launch_grad2e(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles, "
-             "const double* D, double* grad, const double* boys, const float* boysf, double tau, double fp32_tau, "
-             "const double* Dsh, unsigned long long* cnt, int variant, int bs, double tau_prim, double fxs, "
+             "const double* D, const DfBuild& df, double* grad, const double* boys, const float* boysf, double tau, "
+             "double fp32_tau, const double* Dsh, unsigned long long* cnt, int variant, int bs, double tau_prim, double fxs, "
              "cudaStream_t st)")
-    d.append("{ g_tab[cp](P, S, R, tiles, ntiles, D, grad, boys, boysf, tau, fp32_tau, Dsh, cnt, variant, bs, tau_prim, "
+    d.append("{ g_tab[cp](P, S, R, tiles, ntiles, D, df, grad, boys, boysf, tau, fp32_tau, Dsh, cnt, variant, bs, tau_prim, "
              "fxs, st); }")
     d.append("void grad2e_tapes_upload() {")
     for nm in names:

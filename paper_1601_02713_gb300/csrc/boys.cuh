@@ -22,6 +22,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "dfloat.cuh"
+
 #define BOYS_GRID 16          // table points per unit of T
 #define BOYS_TMAX 40.0
 #define BOYS_NT (40 * BOYS_GRID + 1)
@@ -155,6 +157,70 @@ __device__ __forceinline__ void boys_eval(float T, const float* __restrict__ tab
             const float h = 0.5f * it;
 #pragma unroll
             for (int m = 0; m < L; m++) F[m + 1] = ((2 * m + 1) * F[m] - te) * h;
+        }
+    }
+}
+
+// Float-float form (the table is the FP64 one as float-floats, same layout).
+// The Taylor terms from the fourth on are below 2^-24 of the sum and are
+// summed in FP32; each of the others is at most 1/32 of the term it is added
+// to, so Dekker's fast sum applies.
+__device__ __forceinline__ dfloat boys_horner(dfloat f, dfloat x, dfloat t)
+{
+    const dfloat p = f * x, s = fast_two_sum(t.h, p.h);
+    return dfloat(s.h, __fadd_rn(__fadd_rn(s.l, t.l), p.l));
+}
+
+template <int L>
+__device__ __forceinline__ void boys_eval(dfloat T, const dfloat* __restrict__ tab, dfloat theta, dfloat* F)
+{
+    if (T.h < (float)BOYS_TMAX) {
+        const float kf = rintf(T.h * (float)BOYS_GRID);
+        const int k = (int)kf;
+        // T_k and T.h are multiples of ulp(T.h) at most 1/32 apart: exact
+        const dfloat x(__fsub_rn(kf * (1.0f / BOYS_GRID), T.h), -T.l);
+        const dfloat* t = tab + ((size_t)k * BOYS_MT + L) * BOYS_NTAYLOR;
+        float r = ldg(t + 7).h;
+        r = fmaf(r, x.h, ldg(t + 6).h);
+        r = fmaf(r, x.h, ldg(t + 5).h);
+        r = fmaf(r, x.h, ldg(t + 4).h);
+        const dfloat t3 = ldg(t + 3);
+        dfloat f(t3.h, fmaf(r, x.h, t3.l));
+        f = boys_horner(f, x, ldg(t + 2));
+        f = boys_horner(f, x, ldg(t + 1));
+        f = boys_horner(f, x, ldg(t));
+        F[L] = theta * f;
+        if (L > 0) {
+            float e = fmaf(1.0f / 5040.0f, x.h, 1.0f / 720.0f);
+            e = fmaf(e, x.h, 1.0f / 120.0f);
+            e = fmaf(e, x.h, 1.0f / 24.0f);
+            constexpr dfloat c3(1.0 / 6.0);
+            dfloat ex(c3.h, fmaf(e, x.h, c3.l));
+            ex = boys_horner(ex, x, dfloat(0.5f, 0.0f));
+            ex = boys_horner(ex, x, dfloat(1.0f, 0.0f));
+            ex = boys_horner(ex, x, dfloat(1.0f, 0.0f));
+            const dfloat te = theta * ldg(tab + BOYS_EXP_OFF + k) * ex;
+            const dfloat t2(2.0f * T.h, 2.0f * T.l);
+#pragma unroll
+            for (int m = L - 1; m >= 0; m--) F[m] = fma(t2, F[m + 1], te) * dfloat(1.0 / (2 * m + 1));
+        }
+    } else {
+        const dfloat rs = rsqrt_r(T);
+        F[0] = theta * rs * dfloat(0.88622692545275801365);   // sqrt(pi) / 2
+        if (L > 0) {
+            dfloat te(0.0f, 0.0f);
+            if (T.h < (float)BOYS_TEXP) {
+                // e^{-T} is at most 3e-7 of the term it is taken from: e^x - 1 in FP32
+                const float kf = rintf(T.h * (float)BOYS_GRID);
+                const float x = __fsub_rn(kf * (1.0f / BOYS_GRID), T.h) - T.l;
+                float e = fmaf(1.0f / 24.0f, x, 1.0f / 6.0f);
+                e = fmaf(e, x, 0.5f);
+                e = fmaf(e, x, 1.0f);
+                te = theta * ldg(tab + BOYS_EXP_OFF + (int)kf) * dfloat(1.0f, e * x);
+            }
+            const dfloat h = scale2(rs * rs, 0.5f);
+#pragma unroll
+            for (int m = 0; m < L; m++) F[m + 1] = (F[m] * dfloat(2 * m + 1) - te) * h;
         }
     }
 }

@@ -19,6 +19,8 @@
 // which reproduces F = h + J - K/2 with J_mn = sum D_ls (mn|ls) and
 // K_mn = sum D_ls (ml|ns) for a symmetric density.
 #pragma once
+#include <type_traits>
+
 #include "boys.cuh"
 #include "pimd_dev.cuh"
 
@@ -159,6 +161,61 @@ __device__ __forceinline__ void prim_quartet(const R* bra, const R* ket, PrimQ<R
     g.theta = bra[PP_K] * ket[PP_K] * rs;
 }
 
+// The same from float-float pair data. P - Q is formed as AC + (P - A) -
+// (Q - C) with AC the vector between the bra's and the ket's first centre: the
+// differences are exact zeros where the centres coincide (the largest
+// integrals), where the difference of two coordinates would leave 2^-48 of
+// the coordinates themselves. aq = AC - (Q - C), formed once per ket primitive.
+__device__ __forceinline__ void prim_quartet(const dfloat* bra, const dfloat* ket, const dfloat* aq,
+                                             PrimQ<dfloat>& g)
+{
+    const dfloat p = bra[PP_P], q = ket[PP_P];
+    const dfloat rs = rsqrt_r(p + q);
+    const dfloat ipq = rs * rs;
+    const dfloat qi = q * ipq, pi = p * ipq;
+    const dfloat rho = p * qi;
+    dfloat PQ[3];
+#pragma unroll
+    for (int x = 0; x < 3; x++) {
+        g.PA[x] = bra[PP_PAX + x];
+        g.QC[x] = ket[PP_PAX + x];
+        PQ[x] = aq[x] + g.PA[x];
+        g.WP[x] = -(qi * PQ[x]);
+        g.WQ[x] = pi * PQ[x];
+    }
+    g.T = renorm(rho * fma(PQ[0], PQ[0], fma(PQ[1], PQ[1], PQ[2] * PQ[2])));
+    g.o2p = bra[PP_O2P];
+    g.o2pr = rho * bra[PP_O2PP];
+    g.o2q = ket[PP_O2P];
+    g.o2qr = rho * ket[PP_O2PP];
+    g.o2pq = scale2(ipq, 0.5f);
+    g.theta = bra[PP_K] * ket[PP_K] * rs;
+}
+
+__device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ dfloat shfl_xor(dfloat v, int o)
+{
+    return dfloat(__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o));
+}
+
+// sum over the warp, and c v as a double (c a power of two times a sign)
+__device__ __forceinline__ dfloat warp_sum_any(dfloat v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        v += shfl_xor(v, o);
+    return v;
+}
+__device__ __forceinline__ double warp_sum_any(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ double scaled(dfloat v, double c) { return (double)scale2(v, (float)c); }
+__device__ __forceinline__ double scaled(double v, double c) { return c * v; }
+__device__ __forceinline__ double scaled(float v, double c) { return c * (double)v; }
 
 // J'_ab of a tile: every lane of the warp holds a quartet with the same bra
 // pair (ab), so the bra-side Coulomb block sum_cd 2f D_cd (ab|cd) is summed
@@ -174,7 +231,7 @@ __device__ __forceinline__ void bra_coulomb_warp(const R* __restrict__ I, double
 #pragma unroll
     for (int i = 0; i < nc; i++)
 #pragma unroll
-        for (int j = 0; j < nd; j++) Dcd[i * nd + j] = work ? __ldg(D + (size_t)(fc + i) * N + fd + j) : R(0);
+        for (int j = 0; j < nd; j++) Dcd[i * nd + j] = work ? ldg(D + (size_t)(fc + i) * N + fd + j) : R(0);
     const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int a = 0; a < na; a++) {
@@ -185,9 +242,13 @@ __device__ __forceinline__ void bra_coulomb_warp(const R* __restrict__ I, double
             for (int c = 0; c < nc; c++)
 #pragma unroll
                 for (int d = 0; d < nd; d++) s += Dcd[c * nd + d] * I[((a * nb + b) * nc + c) * nd + d];
-            double v = work ? 2.0 * f * (double)s : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            double v;
+            if constexpr (std::is_same<R, dfloat>::value) {
+                // (the weight is a power of two: exact on both parts)
+                v = (double)warp_sum_any(work ? scale2(s, (float)(2.0 * f)) : R(0));
+            } else {
+                v = warp_sum_any(work ? 2.0 * f * (double)s : 0.0);
+            }
             if (lane == 0 && v != 0.0) det_add(G + (size_t)(fa + a) * N + fb + b, v, fxs);
         }
     }
@@ -207,27 +268,27 @@ __device__ __forceinline__ void scatter_jk(const R* __restrict__ I, double f, in
 #pragma unroll
     for (int i = 0; i < na; i++)
 #pragma unroll
-        for (int j = 0; j < nb; j++) Dab[i * nb + j] = __ldg(D + (size_t)(fa + i) * N + fb + j);
+        for (int j = 0; j < nb; j++) Dab[i * nb + j] = ldg(D + (size_t)(fa + i) * N + fb + j);
 #pragma unroll
     for (int i = 0; i < nc; i++)
 #pragma unroll
-        for (int j = 0; j < nd; j++) Dcd[i * nd + j] = __ldg(D + (size_t)(fc + i) * N + fd + j);
+        for (int j = 0; j < nd; j++) Dcd[i * nd + j] = ldg(D + (size_t)(fc + i) * N + fd + j);
 #pragma unroll
     for (int i = 0; i < na; i++)
 #pragma unroll
-        for (int j = 0; j < nc; j++) Dac[i * nc + j] = __ldg(D + (size_t)(fa + i) * N + fc + j);
+        for (int j = 0; j < nc; j++) Dac[i * nc + j] = ldg(D + (size_t)(fa + i) * N + fc + j);
 #pragma unroll
     for (int i = 0; i < na; i++)
 #pragma unroll
-        for (int j = 0; j < nd; j++) Dad[i * nd + j] = __ldg(D + (size_t)(fa + i) * N + fd + j);
+        for (int j = 0; j < nd; j++) Dad[i * nd + j] = ldg(D + (size_t)(fa + i) * N + fd + j);
 #pragma unroll
     for (int i = 0; i < nb; i++)
 #pragma unroll
-        for (int j = 0; j < nc; j++) Dbc[i * nc + j] = __ldg(D + (size_t)(fb + i) * N + fc + j);
+        for (int j = 0; j < nc; j++) Dbc[i * nc + j] = ldg(D + (size_t)(fb + i) * N + fc + j);
 #pragma unroll
     for (int i = 0; i < nb; i++)
 #pragma unroll
-        for (int j = 0; j < nd; j++) Dbd[i * nd + j] = __ldg(D + (size_t)(fb + i) * N + fd + j);
+        for (int j = 0; j < nd; j++) Dbd[i * nd + j] = ldg(D + (size_t)(fb + i) * N + fd + j);
 
     // J'_ab (rows of the bra)
     if (bra_j) {
@@ -240,7 +301,7 @@ __device__ __forceinline__ void scatter_jk(const R* __restrict__ I, double f, in
                 for (int c = 0; c < nc; c++)
 #pragma unroll
                     for (int d = 0; d < nd; d++) s += Dcd[c * nd + d] * I[((a * nb + b) * nc + c) * nd + d];
-                det_add(G + (size_t)(fa + a) * N + fb + b, 2.0 * f * (double)s, fxs);
+                det_add(G + (size_t)(fa + a) * N + fb + b, scaled(s, 2.0 * f), fxs);
             }
         }
     }
@@ -253,7 +314,7 @@ __device__ __forceinline__ void scatter_jk(const R* __restrict__ I, double f, in
             for (int a = 0; a < na; a++)
 #pragma unroll
                 for (int b = 0; b < nb; b++) s += Dab[a * nb + b] * I[((a * nb + b) * nc + c) * nd + d];
-            det_add(G + (size_t)(fc + c) * N + fd + d, 2.0 * f * (double)s, fxs);
+            det_add(G + (size_t)(fc + c) * N + fd + d, scaled(s, 2.0 * f), fxs);
         }
 #pragma unroll
     for (int a = 0; a < na; a++)
@@ -264,7 +325,7 @@ __device__ __forceinline__ void scatter_jk(const R* __restrict__ I, double f, in
             for (int b = 0; b < nb; b++)
 #pragma unroll
                 for (int d = 0; d < nd; d++) s += Dbd[b * nd + d] * I[((a * nb + b) * nc + c) * nd + d];
-            det_add(G + (size_t)(fa + a) * N + fc + c, -0.5 * f * (double)s, fxs);
+            det_add(G + (size_t)(fa + a) * N + fc + c, scaled(s, -0.5 * f), fxs);
         }
 #pragma unroll
     for (int b = 0; b < nb; b++)
@@ -275,7 +336,7 @@ __device__ __forceinline__ void scatter_jk(const R* __restrict__ I, double f, in
             for (int a = 0; a < na; a++)
 #pragma unroll
                 for (int d = 0; d < nd; d++) s += Dad[a * nd + d] * I[((a * nb + b) * nc + c) * nd + d];
-            det_add(G + (size_t)(fb + b) * N + fc + c, -0.5 * f * (double)s, fxs);
+            det_add(G + (size_t)(fb + b) * N + fc + c, scaled(s, -0.5 * f), fxs);
         }
 #pragma unroll
     for (int a = 0; a < na; a++)
@@ -286,7 +347,7 @@ __device__ __forceinline__ void scatter_jk(const R* __restrict__ I, double f, in
             for (int b = 0; b < nb; b++)
 #pragma unroll
                 for (int c = 0; c < nc; c++) s += Dbc[b * nc + c] * I[((a * nb + b) * nc + c) * nd + d];
-            det_add(G + (size_t)(fa + a) * N + fd + d, -0.5 * f * (double)s, fxs);
+            det_add(G + (size_t)(fa + a) * N + fd + d, scaled(s, -0.5 * f), fxs);
         }
 #pragma unroll
     for (int b = 0; b < nb; b++)
@@ -297,7 +358,7 @@ __device__ __forceinline__ void scatter_jk(const R* __restrict__ I, double f, in
             for (int a = 0; a < na; a++)
 #pragma unroll
                 for (int c = 0; c < nc; c++) s += Dac[a * nc + c] * I[((a * nb + b) * nc + c) * nd + d];
-            det_add(G + (size_t)(fb + b) * N + fd + d, -0.5 * f * (double)s, fxs);
+            det_add(G + (size_t)(fb + b) * N + fd + d, scaled(s, -0.5 * f), fxs);
         }
 }
 
@@ -314,6 +375,13 @@ __device__ __forceinline__ void load_ppn(const Pairs& P, int g, int k, float* ou
 #pragma unroll
     for (int f = 0; f < nf; f++) out[f] = __ldg(P.ppf + ((size_t)f * PIMD_MAXPP + k) * n + g);
 }
+__device__ __forceinline__ void load_ppn(const Pairs& P, int g, int k, dfloat* out, int nf)
+{
+    const size_t n = P.n;
+#pragma unroll
+    for (int f = 0; f < nf; f++) out[f] = ldg(P.ppd + ((size_t)f * PIMD_MAXPP + k) * n + g);
+}
+__device__ __forceinline__ const dfloat* pp_base(const Pairs& P, dfloat) { return P.ppd; }
 __device__ __forceinline__ const double* pp_base(const Pairs& P, double) { return P.pp; }
 __device__ __forceinline__ const float* pp_base(const Pairs& P, float) { return P.ppf; }
 
@@ -348,48 +416,80 @@ __device__ __forceinline__ int stair_total(const float* sqp, int nbra, const Pai
     return total;
 }
 
+// S lanes of a warp (S a power of two, sub = 0..S-1 of this one) share a
+// quartet: each takes every S-th position of the sequence, and the
+// contracted accumulators are summed over them before the horizontal
+// recursion. Every lane of the warp calls this (total = 0: no quartet; cd then
+// any pair); kmax: the longest sequence of the warp.
 template <class C, typename R>
-__device__ __forceinline__ int quartet_cart(const R (*sbra)[PIMD_MAXPP], const float* sqp, int nbra, const Pairs& P,
-                                            int cd, const double A[3], const double B[3], const double Cc[3],
-                                            const double Dd[3], const R* __restrict__ boys, float qthr, int total,
-                                            int kmax, R* cart)
+__device__ __forceinline__ void quartet_cart(const R (*sbra)[PIMD_MAXPP], const float* sqp, int nbra, const Pairs& P,
+                                             int cd, const R AB[3], const R CD[3], const R AC[3],
+                                             const R* __restrict__ boys, float qthr, int total, int kmax, int S,
+                                             int sub, R* cart)
 {
+    constexpr bool DF = std::is_same<R, dfloat>::value;
     R acc[C::NE * C::NF];
 #pragma unroll
     for (int i = 0; i < C::NE * C::NF; i++) acc[i] = R(0);
-    const int nket = P.npp[cd];
-    int i = 0, j = 0;
+    // position `pos` of the sequence = bra primitive i of ket primitive j,
+    // whose row is w long
+    int i = sub, j = 0, jl = -1;
     int w = total > 0 ? (qthr > 0.0f ? stair_width(sqp, nbra, __ldg(P.qp + cd), qthr) : nbra) : 0;
-    R ket[PP_NERI];
-    for (int k = 0; k < kmax; k++) {
-        if (k < total) {
-            if (i == 0) load_ppn(P, cd, j, ket, PP_NERI);
+    R ket[PP_NERI], aq[3];
+    for (int k = 0; k < kmax; k += S) {
+        if (k + sub < total) {
+            while (i >= w) {
+                i -= w;
+                j++;
+                if (qthr > 0.0f) w = stair_width(sqp, nbra, __ldg(P.qp + (size_t)j * P.n + cd), qthr);
+            }
+            if (j != jl) {
+                load_ppn(P, cd, j, ket, PP_NERI);
+                jl = j;
+                if constexpr (DF)
+#pragma unroll
+                    for (int x = 0; x < 3; x++) aq[x] = AC[x] - ket[PP_PAX + x];
+            }
             R bra[PP_NERI];
 #pragma unroll
             for (int f = 0; f < PP_NERI; f++) bra[f] = sbra[f][i];
             PrimQ<R> g;
-            prim_quartet<R>(bra, ket, g);
+            if constexpr (DF)
+                prim_quartet(bra, ket, aq, g);
+            else
+                prim_quartet<R>(bra, ket, g);
             R F[C::L + 1];
             boys_eval<C::L>(g.T, boys, g.theta, F);
             C::template vrr<R>(F, g.PA[0], g.PA[1], g.PA[2], g.WP[0], g.WP[1], g.WP[2], g.QC[0], g.QC[1], g.QC[2],
                                g.WQ[0], g.WQ[1], g.WQ[2], g.o2p, g.o2pr, g.o2q, g.o2qr, g.o2pq, acc);
-            if (++i == w) {
-                i = 0;
-                if (++j < nket)
-                    w = qthr > 0.0f ? stair_width(sqp, nbra, __ldg(P.qp + (size_t)j * P.n + cd), qthr) : nbra;
-            }
+            i += S;
         }
     }
-    C::template hrr<R>(acc, R(A[0] - B[0]), R(A[1] - B[1]), R(A[2] - B[2]), R(Cc[0] - Dd[0]), R(Cc[1] - Dd[1]),
-                       R(Cc[2] - Dd[2]), cart);
-    return total;
+    for (int o = 1; o < S; o <<= 1)
+#pragma unroll
+        for (int e = 0; e < C::NE * C::NF; e++) acc[e] += shfl_xor(acc[e], o);
+    if (sub == 0) C::template hrr<R>(acc, AB[0], AB[1], AB[2], CD[0], CD[1], CD[2], cart);
+}
+
+// Blocks per tile of the straight-line kernels (gridDim.y): a block takes every
+// gridDim.y-th of the tile's quartets and, where few are left to it, several
+// lanes per quartet, so a small batch's primitive loops are spread over the
+// chip instead of running 81 recursions deep on a few warps. Batches with two
+// blocks of 128 threads per SM already fill the register files.
+// With the float-float kernels: the Fock build of one water molecule 18.8 ->
+// 6.3 ms, the forces of 4 minimal-basis dimers 37.3 -> 12.5 ms, of one (H2O)8
+// bead 1196 -> 843 ms.
+inline int jk_blocks_per_tile(int ntiles)
+{
+    const int want = 4 * 152;
+    return ntiles >= want ? 1 : (want + ntiles - 1) / ntiles < 8 ? (want + ntiles - 1) / ntiles : 8;
 }
 
 // tau_prim: primitive quartets whose bound qp_i qp_j (density bound) is below
 // it are skipped (0 keeps every primitive quartet). fxs > 0: G' accumulated as
 // fixed-point integers (det_add).
 template <class C, typename R>
-__global__ void __launch_bounds__(128) jk_kernel(Pairs P, Shells S, Reps R_, const Tile* __restrict__ tiles,
+__global__ void __launch_bounds__(128) jk_kernel(Pairs P, Shells S_, Reps R_, const Tile* __restrict__ tiles,
                                                  const R* __restrict__ Dall, double* __restrict__ Gall,
                                                  const R* __restrict__ boys, double tau_lo, double tau_hi,
                                                  const double* __restrict__ Dsh, unsigned long long* __restrict__ cnt,
@@ -402,7 +502,7 @@ __global__ void __launch_bounds__(128) jk_kernel(Pairs P, Shells S, Reps R_, con
     const int ab = t.ab;
     for (int e = threadIdx.x; e < PP_NERI * PIMD_MAXPP; e += blockDim.x) {
         const int f = e / PIMD_MAXPP, k = e % PIMD_MAXPP;
-        sbra[f][k] = pp_base(P, R(0))[((size_t)f * PIMD_MAXPP + k) * P.n + ab];
+        sbra[f][k] = pp_base(P, R())[((size_t)f * PIMD_MAXPP + k) * P.n + ab];
     }
     if (threadIdx.x < PIMD_MAXPP) sqp[threadIdx.x] = P.qp[(size_t)threadIdx.x * P.n + ab];
     __syncthreads();
@@ -429,55 +529,69 @@ __global__ void __launch_bounds__(128) jk_kernel(Pairs P, Shells S, Reps R_, con
     int cd, sc, sd;
     float qthr;
     bool work = screen(threadIdx.x, cd, sc, sd, qthr);
-    if (tau_prim > 0.0 && blockDim.x > 32) {
-        // Lanes stop their primitive loops at their own cutoff, and a warp
-        // issues for all its lanes: the block's quartets are regrouped by the
-        // number of primitive quartets that survive (descending, bitonic sort
-        // over the block), so that a warp holds quartets of similar length.
-        __shared__ int skey[128], sidx[128];
-        const int est = work ? stair_total(sqp, nbra, P, cd, qthr) : -1;
-        const int tid = threadIdx.x, bd = blockDim.x;
-        skey[tid] = est;
-        sidx[tid] = tid;
-        __syncthreads();
-        for (int k = 2; k <= bd; k <<= 1)
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                const int o = tid ^ j;
-                if (o > tid) {
-                    const bool desc = (tid & k) == 0;
-                    const int a = skey[tid], b = skey[o];
-                    if (desc ? a < b : a > b) {
-                        skey[tid] = b;
-                        skey[o] = a;
-                        const int x = sidx[tid];
-                        sidx[tid] = sidx[o];
-                        sidx[o] = x;
-                    }
+    const int tid = threadIdx.x, bd = blockDim.x;
+    // quartets of the tile that are left, and this block's share of them
+    const int nwork = __syncthreads_count(work);
+    const int mine = (nwork - (int)blockIdx.y + (int)gridDim.y - 1) / (int)gridDim.y;
+    if (mine <= 0) return;
+    // Lanes stop their primitive loops at their own cutoff, and a warp issues
+    // for all its lanes: the tile's quartets are regrouped by the number of
+    // primitive quartets that survive (descending, bitonic sort over the
+    // block; the ones screened out last), so that a warp holds quartets of
+    // similar length. Lanes without a quartet of their own are given to the
+    // others, S to a quartet; the FP32 quartets keep one lane each, and with it
+    // the order of their sums.
+    __shared__ int skey[128], sidx[128];
+    skey[tid] = work ? stair_total(sqp, nbra, P, cd, qthr) : -1;
+    sidx[tid] = tid;
+    __syncthreads();
+    for (int k = 2; k <= bd; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const int o = tid ^ j;
+            if (o > tid) {
+                const bool desc = (tid & k) == 0;
+                const int a = skey[tid], b = skey[o];
+                if (desc ? a < b : a > b) {
+                    skey[tid] = b;
+                    skey[o] = a;
+                    const int x = sidx[tid];
+                    sidx[tid] = sidx[o];
+                    sidx[o] = x;
                 }
-                __syncthreads();
             }
-        work = screen(sidx[tid], cd, sc, sd, qthr);
-    }
+            __syncthreads();
+        }
+    int S = 1;
+    if constexpr (!std::is_same<R, float>::value)
+        while (S < 32 && 2 * S * mine <= bd) S *= 2;
+    const int item = tid / S, sub = tid % S;
+    work = item < mine && screen(sidx[blockIdx.y + item * gridDim.y], cd, sc, sd, qthr);
     const int sa = P.sa[ab], sb = P.sb[ab];
     // a warp with no quartet left leaves; otherwise every lane stays for the
-    // warp-wide J'_ab sum (the block's warps share the bra pair)
+    // sums over lanes (the block's warps share the bra pair)
     if (__all_sync(0xffffffffu, !work)) return;
     constexpr int NCART = ncart(C::LA) * ncart(C::LB) * ncart(C::LC) * ncart(C::LD);
     R cart[NCART], tmp[NCART];
-    double f = 0.0;
-    int nprim = 0;
     const int total = work ? stair_total(sqp, nbra, P, cd, qthr) : 0;
     const int kmax = __reduce_max_sync(0xffffffffu, (unsigned)total);
+    R AB[3], CD[3], AC[3];
     if (work) {
-        double A[3], B[3], Cc[3], Dd[3];
 #pragma unroll
         for (int x = 0; x < 3; x++) {
-            A[x] = S.xyz[3 * sa + x];
-            B[x] = S.xyz[3 * sb + x];
-            Cc[x] = S.xyz[3 * sc + x];
-            Dd[x] = S.xyz[3 * sd + x];
+            if constexpr (std::is_same<R, dfloat>::value) {
+                AB[x] = ldg(P.abd + (size_t)x * P.n + ab);
+                CD[x] = ldg(P.abd + (size_t)x * P.n + cd);
+                AC[x] = ldg(S_.xyzd + 3 * sa + x) - ldg(S_.xyzd + 3 * sc + x);
+            } else {
+                AB[x] = R(S_.xyz[3 * sa + x] - S_.xyz[3 * sb + x]);
+                CD[x] = R(S_.xyz[3 * sc + x] - S_.xyz[3 * sd + x]);
+            }
         }
-        nprim = quartet_cart<C, R>(sbra, sqp, nbra, P, cd, A, B, Cc, Dd, boys, qthr, total, kmax, cart);
+    }
+    quartet_cart<C, R>(sbra, sqp, nbra, P, cd, AB, CD, AC, boys, qthr, total, kmax, S, sub, cart);
+    work = work && sub == 0;
+    double f = 0.0;
+    if (work) {
         cart_to_sph4<C::LA, C::LB, C::LC, C::LD>(cart, tmp);
         f = 1.0;
         if (sa == sb) f *= 0.5;
@@ -485,7 +599,7 @@ __global__ void __launch_bounds__(128) jk_kernel(Pairs P, Shells S, Reps R_, con
         if (ab == cd) f *= 0.5;
     }
     const unsigned nq = __reduce_add_sync(0xffffffffu, work ? 1u : 0u);
-    const unsigned np = __reduce_add_sync(0xffffffffu, (unsigned)nprim);
+    const unsigned np = __reduce_add_sync(0xffffffffu, work ? (unsigned)total : 0u);
     if ((threadIdx.x & 31) == 0 && nq) {
         atomicAdd(cnt, (unsigned long long)nq);
         atomicAdd(cnt + 1, (unsigned long long)np);
@@ -493,10 +607,10 @@ __global__ void __launch_bounds__(128) jk_kernel(Pairs P, Shells S, Reps R_, con
     }
     const int N = R_.nbf[r];
     const size_t off = R_.moff[r];
-    bra_coulomb_warp<C::LA, C::LB, C::LC, C::LD, R>(cart, f, work, S.bf[P.sa[ab]], S.bf[P.sb[ab]], S.bf[sc],
-                                                     S.bf[sd], N, Dall + off, Gall + off, fxs);
+    bra_coulomb_warp<C::LA, C::LB, C::LC, C::LD, R>(cart, f, work, S_.bf[P.sa[ab]], S_.bf[P.sb[ab]], S_.bf[sc],
+                                                     S_.bf[sd], N, Dall + off, Gall + off, fxs);
     if (work)
-        scatter_jk<C::LA, C::LB, C::LC, C::LD, R>(cart, f, S.bf[sa], S.bf[sb], S.bf[sc], S.bf[sd], N, Dall + off,
+        scatter_jk<C::LA, C::LB, C::LC, C::LD, R>(cart, f, S_.bf[sa], S_.bf[sb], S_.bf[sc], S_.bf[sd], N, Dall + off,
                                                   Gall + off, fxs, false);
 }
 

@@ -529,6 +529,18 @@ def encode_hrr(op):
 COOP_ENERGY_MIN_VRR = 2000
 STRAIGHT_ENERGY_MAX_VRR = 2000
 COOP_GRAD_MIN_VRR = 400
+# float-float Fock kernel (dfloat.cuh): up to this many operations per
+# primitive quartet. A multiply-add is 12 FP32 instructions, and above this the
+# recursion's code (tens of kilobytes) no longer stays in the instruction
+# caches: 8 (H2O)8 beads, one build, FP64 -> float-float: (ps|ss) 36.7 -> 5.2 ms,
+# (pp|ps) 51.6 -> 12.3, (dp|ps) 41.5 -> 17.7, (dp|ds), the largest in, 32.7 ->
+# 23.8; (dp|pp), the smallest out, 51.7 -> 61.3, (dp|dp) 39.3 -> 62.5.
+DF_MAX_FLOPS = 1600
+# the gradient's recursion runs to order L + 1 into four accumulator sets, so its
+# code and registers reach the limit sooner: one bead, FP64 -> float-float:
+# (ps|ss) 8.5 -> 3.0 ms, (ps|ps) 13.6 -> 4.9, (dp|ss), the largest in, 5.3 ->
+# 4.3; (ds|ps), the smallest out, 11.6 -> 11.7, (pp|ps) 24.1 -> 87.4.
+DF_GRAD_MAX_FLOPS = 900
 
 
 def _sort_levels(ops, base_level):
@@ -853,7 +865,8 @@ def generate(outdir):
         if coop_g:
             hdr, _ = coop_header(nm, True, gen_coop(c, True))
             write_if_changed(os.path.join(outdir, f"coopg_{nm}.cuh"), hdr)
-        stats.append((nm, nl, nfl, nh, gnl, gnfl, heavy, coop_e, coop_g, straight_e))
+        stats.append((nm, nl, nfl, nh, gnl, gnfl, heavy, coop_e, coop_g, straight_e, straight_e and nfl <= DF_MAX_FLOPS,
+                      not heavy and gnfl <= DF_GRAD_MAX_FLOPS))
     return stats
 
 

@@ -39,23 +39,28 @@ __device__ __forceinline__ int cidx(int lx, int ly, int lz)
     return (l - lx) * (l - lx + 1) / 2 + lz;
 }
 
-// Gamma of one quartet in Cartesian components: Gc[((a*nb+b)*nc+c)*nd+d]
-template <int LA, int LB, int LC, int LD, typename R = double>
+// Gamma of one quartet in Cartesian components: Gc[((a*nb+b)*nc+c)*nd+d], from
+// a density in FP64, or for the float-float kernels in float-float (TD)
+template <int LA, int LB, int LC, int LD, typename R = double, typename TD = double>
 __device__ __forceinline__ void gamma_cart(double f, int fa, int fb, int fc, int fd, int N,
-                                           const double* __restrict__ D, R* Gc, R* tmp)
+                                           const TD* __restrict__ D, R* Gc, R* tmp)
 {
     constexpr int na = nsph(LA), nb = nsph(LB), nc = nsph(LC), nd = nsph(LD);
     for (int a = 0; a < na; a++)
         for (int b = 0; b < nb; b++) {
-            const double dab = __ldg(D + (size_t)(fa + a) * N + fb + b);
+            const TD dab = ldg(D + (size_t)(fa + a) * N + fb + b);
             for (int c = 0; c < nc; c++) {
-                const double dac = __ldg(D + (size_t)(fa + a) * N + fc + c);
-                const double dbc = __ldg(D + (size_t)(fb + b) * N + fc + c);
+                const TD dac = ldg(D + (size_t)(fa + a) * N + fc + c);
+                const TD dbc = ldg(D + (size_t)(fb + b) * N + fc + c);
                 for (int d = 0; d < nd; d++) {
-                    const double dcd = __ldg(D + (size_t)(fc + c) * N + fd + d);
-                    const double dbd = __ldg(D + (size_t)(fb + b) * N + fd + d);
-                    const double dad = __ldg(D + (size_t)(fa + a) * N + fd + d);
-                    Gc[((a * nb + b) * nc + c) * nd + d] = R(f * (4.0 * dab * dcd - dac * dbd - dad * dbc));
+                    const TD dcd = ldg(D + (size_t)(fc + c) * N + fd + d);
+                    const TD dbd = ldg(D + (size_t)(fb + b) * N + fd + d);
+                    const TD dad = ldg(D + (size_t)(fa + a) * N + fd + d);
+                    if constexpr (std::is_same<R, dfloat>::value)
+                        Gc[((a * nb + b) * nc + c) * nd + d] =
+                            scale2(scale2(dab * dcd, 4.0f) - dac * dbd - dad * dbc, (float)f);
+                    else
+                        Gc[((a * nb + b) * nc + c) * nd + d] = R(f * (4.0 * dab * dcd - dac * dbd - dad * dbc));
                 }
             }
         }
@@ -94,7 +99,7 @@ __device__ __forceinline__ void contract_deriv(const R* Gc, Up up, Dn dn, R g[3]
                             ed[x]--;
                             int jd[4] = {i0, i1, i2, i3};
                             jd[POS] = cidx(ed[0], ed[1], ed[2]);
-                            v -= e[x] * dn(((jd[0] * ndn[1] + jd[1]) * ndn[2] + jd[2]) * ndn[3] + jd[3]);
+                            v -= R(e[x]) * dn(((jd[0] * ndn[1] + jd[1]) * ndn[2] + jd[2]) * ndn[3] + jd[3]);
                         }
                         g[x] += gm * v;
                     }
@@ -115,7 +120,7 @@ __device__ __forceinline__ void scatter_grad(double* grad, const Shells& S, int 
     const int aa = S.atom[sa], ab = S.atom[sb], ac = S.atom[sc], ad = S.atom[sd];
 #pragma unroll
     for (int x = 0; x < 3; x++) {
-        const double a = gA[x], b = gB[x], c = gC[x];
+        const double a = (double)gA[x], b = (double)gB[x], c = (double)gC[x];
         det_add(grad + 3 * aa + x, a, fxs);
         det_add(grad + 3 * ab + x, b, fxs);
         det_add(grad + 3 * ac + x, c, fxs);
@@ -138,11 +143,21 @@ __device__ __forceinline__ double gamma_bound(const Reps& R, const double* Dsh, 
 // Primitive screening: primitive quartet (i|j) is skipped when
 // (qg_i qp_j + qp_i qg_j) |Gamma| < tau_prim (qg: the derivative scale of a
 // primitive pair); tau_prim = 0 keeps every primitive quartet.
+// the density a gradient kernel of precision R reads
+template <typename R>
+struct GradDensity {
+    typedef double T;
+};
+template <>
+struct GradDensity<dfloat> {
+    typedef dfloat T;
+};
+
 template <class G, typename R>
 __global__ void __launch_bounds__(128) grad2e_kernel(Pairs P, Shells S, Reps Rp, const Tile* __restrict__ tiles,
-                                                     const double* __restrict__ Dall, double* __restrict__ grad,
-                                                     const R* __restrict__ boys, double tau_lo, double tau_hi,
-                                                     const double* __restrict__ Dsh,
+                                                     const typename GradDensity<R>::T* __restrict__ Dall,
+                                                     double* __restrict__ grad, const R* __restrict__ boys, double tau_lo,
+                                                     double tau_hi, const double* __restrict__ Dsh,
                                                      unsigned long long* __restrict__ cnt, double tau_prim,
                                                      double fxs)
 {
@@ -153,7 +168,7 @@ __global__ void __launch_bounds__(128) grad2e_kernel(Pairs P, Shells S, Reps Rp,
     const int ab = t.ab;
     for (int e = threadIdx.x; e < PP_NF * PIMD_MAXPP; e += blockDim.x) {
         const int f = e / PIMD_MAXPP, k = e % PIMD_MAXPP;
-        sbra[f][k] = pp_base(P, R(0))[((size_t)f * PIMD_MAXPP + k) * P.n + ab];
+        sbra[f][k] = pp_base(P, R())[((size_t)f * PIMD_MAXPP + k) * P.n + ab];
     }
     if (threadIdx.x < PIMD_MAXPP) {
         sqp[threadIdx.x] = P.qp[(size_t)threadIdx.x * P.n + ab];
@@ -178,42 +193,47 @@ __global__ void __launch_bounds__(128) grad2e_kernel(Pairs P, Shells S, Reps Rp,
     double gam;
     float gthr;
     bool work = screen(threadIdx.x, cd, gam, gthr);
-    if (tau_prim > 0.0 && blockDim.x > 32) {
-        // regroup the block's quartets by their number of surviving primitive
-        // quartets (bitonic sort, descending): lanes stop at their own cutoff
-        // and a warp issues for all its lanes
-        __shared__ int skey[128], sidx[128];
-        int est = -1;
-        if (work) {
-            est = 0;
-            const int nket = P.npp[cd];
-            for (int j = 0; j < nket; j++) {
-                const float qpj = __ldg(P.qp + (size_t)j * P.n + cd), qgj = __ldg(P.qg + (size_t)j * P.n + cd);
-                for (int i = 0; i < nbra; i++) est += sqg[i] * qpj + sqp[i] * qgj >= gthr;
-            }
+    const int tid = threadIdx.x, bd = blockDim.x;
+    const int nwork = __syncthreads_count(work);
+    const int mine = (nwork - (int)blockIdx.y + (int)gridDim.y - 1) / (int)gridDim.y;
+    if (mine <= 0) return;
+    // regroup the tile's quartets by their number of surviving primitive
+    // quartets and give spare lanes to quartets, as in jk_kernel
+    __shared__ int skey[128], sidx[128];
+    int est = -1;
+    if (work) {
+        est = 0;
+        const int nket = P.npp[cd];
+        for (int j = 0; j < nket; j++) {
+            const float qpj = __ldg(P.qp + (size_t)j * P.n + cd), qgj = __ldg(P.qg + (size_t)j * P.n + cd);
+            for (int i = 0; i < nbra; i++) est += sqg[i] * qpj + sqp[i] * qgj >= gthr;
         }
-        const int tid = threadIdx.x, bd = blockDim.x;
-        skey[tid] = est;
-        sidx[tid] = tid;
-        __syncthreads();
-        for (int k = 2; k <= bd; k <<= 1)
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                const int o = tid ^ j;
-                if (o > tid) {
-                    const bool desc = (tid & k) == 0;
-                    const int a = skey[tid], b = skey[o];
-                    if (desc ? a < b : a > b) {
-                        skey[tid] = b;
-                        skey[o] = a;
-                        const int x = sidx[tid];
-                        sidx[tid] = sidx[o];
-                        sidx[o] = x;
-                    }
-                }
-                __syncthreads();
-            }
-        work = screen(sidx[tid], cd, gam, gthr);
     }
+    skey[tid] = est;
+    sidx[tid] = tid;
+    __syncthreads();
+    for (int k = 2; k <= bd; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const int o = tid ^ j;
+            if (o > tid) {
+                const bool desc = (tid & k) == 0;
+                const int a = skey[tid], b = skey[o];
+                if (desc ? a < b : a > b) {
+                    skey[tid] = b;
+                    skey[o] = a;
+                    const int x = sidx[tid];
+                    sidx[tid] = sidx[o];
+                    sidx[o] = x;
+                }
+            }
+            __syncthreads();
+        }
+    int S_ = 1;
+    if constexpr (!std::is_same<R, float>::value)
+        while (S_ < 32 && 2 * S_ * mine <= bd) S_ *= 2;
+    const int lanes = S_, item = tid / lanes, sub = tid % lanes;
+    work = item < mine && screen(sidx[blockIdx.y + item * gridDim.y], cd, gam, gthr);
+    if (__all_sync(0xffffffffu, !work)) return;
     // the lane's surviving primitive quartets, walked as one flat sequence
     // (row-major over (j, i)) for kmax steps, kmax the longest of the warp
     auto survives = [&](int i, float qpj, float qgj) { return sqg[i] * qpj + sqp[i] * qgj >= gthr; };
@@ -228,36 +248,44 @@ __global__ void __launch_bounds__(128) grad2e_kernel(Pairs P, Shells S, Reps Rp,
     const int kmax = __reduce_max_sync(0xffffffffu, (unsigned)total);
     {
         // executed quartets and primitive quartets (one atomic pair per warp)
-        const unsigned nq = __reduce_add_sync(0xffffffffu, work ? 1u : 0u);
-        const unsigned np = __reduce_add_sync(0xffffffffu, (unsigned)total);
+        const unsigned nq = __reduce_add_sync(0xffffffffu, work && sub == 0 ? 1u : 0u);
+        const unsigned np = __reduce_add_sync(0xffffffffu, sub == 0 ? (unsigned)total : 0u);
         if ((threadIdx.x & 31) == 0 && nq) {
             atomicAdd(cnt, (unsigned long long)nq);
             atomicAdd(cnt + 1, (unsigned long long)np);
         }
     }
-    if (!work) return;
-    const int sc = P.sa[cd], sd = P.sb[cd];
-    double A[3], B[3], Cc[3], Dd[3];
+    constexpr bool DF = std::is_same<R, dfloat>::value;
+    const int sc = work ? P.sa[cd] : sa, sd = work ? P.sb[cd] : sb;
+    R AB[3], CD[3], AC[3];
 #pragma unroll
     for (int x = 0; x < 3; x++) {
-        A[x] = S.xyz[3 * sa + x];
-        B[x] = S.xyz[3 * sb + x];
-        Cc[x] = S.xyz[3 * sc + x];
-        Dd[x] = S.xyz[3 * sd + x];
+        if constexpr (DF) {
+            AB[x] = ldg(P.abd + (size_t)x * P.n + ab);
+            CD[x] = ldg(P.abd + (size_t)x * P.n + (work ? cd : ab));
+            AC[x] = ldg(S.xyzd + 3 * sa + x) - ldg(S.xyzd + 3 * sc + x);
+        } else {
+            AB[x] = R(S.xyz[3 * sa + x] - S.xyz[3 * sb + x]);
+            CD[x] = R(S.xyz[3 * sc + x] - S.xyz[3 * sd + x]);
+        }
     }
     R accU[G::N_accU], accA[G::N_accA], accB[G::N_accB], accC[G::N_accC];
     for (int i = 0; i < G::N_accU; i++) accU[i] = R(0);
     for (int i = 0; i < G::N_accA; i++) accA[i] = R(0);
     for (int i = 0; i < G::N_accB; i++) accB[i] = R(0);
     for (int i = 0; i < G::N_accC; i++) accC[i] = R(0);
-    const int nket = P.npp[cd];
-    int i = 0, j = 0, jl = -1;
-    float qpj = __ldg(P.qp + cd), qgj = __ldg(P.qg + cd);
-    R ket[PP_NF];
-    for (int k = 0; k < kmax; k++) {
-        if (k < total) {
-            // advance to the next surviving primitive quartet (one exists: k < total)
-            while (!survives(i, qpj, qgj)) {
+    int i = 0, j = 0, jl = -1, skip = sub;   // survivors to pass over before this lane's next one
+    float qpj = 0.0f, qgj = 0.0f;
+    if (work) {
+        qpj = __ldg(P.qp + cd);
+        qgj = __ldg(P.qg + cd);
+    }
+    R ket[PP_NF], aq[3];
+    for (int k = 0; k < kmax; k += lanes) {
+        if (k + sub < total) {
+            // advance to this lane's next surviving primitive quartet (one exists: k + sub < total)
+            while (true) {
+                if (survives(i, qpj, qgj) && skip-- == 0) break;
                 if (++i == nbra) {
                     i = 0;
                     ++j;
@@ -265,30 +293,37 @@ __global__ void __launch_bounds__(128) grad2e_kernel(Pairs P, Shells S, Reps Rp,
                     qgj = __ldg(P.qg + (size_t)j * P.n + cd);
                 }
             }
+            skip = lanes;   // the one evaluated now is the first passed over
             if (j != jl) {
                 load_ppn(P, cd, j, ket, PP_NF);
                 jl = j;
+                if constexpr (DF)
+#pragma unroll
+                    for (int x = 0; x < 3; x++) aq[x] = AC[x] - ket[PP_PAX + x];
             }
             R bra[PP_NERI];
 #pragma unroll
             for (int f = 0; f < PP_NERI; f++) bra[f] = sbra[f][i];
             PrimQ<R> g;
-            prim_quartet<R>(bra, ket, g);
+            if constexpr (DF)
+                prim_quartet(bra, ket, aq, g);
+            else
+                prim_quartet<R>(bra, ket, g);
             R F[G::L + 1];
             boys_eval<G::L>(g.T, boys, g.theta, F);
             G::template vrr<R>(F, g.PA[0], g.PA[1], g.PA[2], g.WP[0], g.WP[1], g.WP[2], g.QC[0], g.QC[1], g.QC[2],
                                g.WQ[0], g.WQ[1], g.WQ[2], g.o2p, g.o2pr, g.o2q, g.o2qr, g.o2pq, accU, accA, accB,
                                accC, R(2) * sbra[PP_EA][i], R(2) * sbra[PP_EB][i], R(2) * ket[PP_EA]);
-            if (++i == nbra && j + 1 < nket) {
-                i = 0;
-                ++j;
-                qpj = __ldg(P.qp + (size_t)j * P.n + cd);
-                qgj = __ldg(P.qg + (size_t)j * P.n + cd);
-            }
         }
     }
-    const R AB0 = R(A[0] - B[0]), AB1 = R(A[1] - B[1]), AB2 = R(A[2] - B[2]);
-    const R CD0 = R(Cc[0] - Dd[0]), CD1 = R(Cc[1] - Dd[1]), CD2 = R(Cc[2] - Dd[2]);
+    for (int o = 1; o < lanes; o <<= 1) {
+        for (int e = 0; e < G::N_accU; e++) accU[e] += shfl_xor(accU[e], o);
+        for (int e = 0; e < G::N_accA; e++) accA[e] += shfl_xor(accA[e], o);
+        for (int e = 0; e < G::N_accB; e++) accB[e] += shfl_xor(accB[e], o);
+        for (int e = 0; e < G::N_accC; e++) accC[e] += shfl_xor(accC[e], o);
+    }
+    if (!work || sub != 0) return;
+    const R AB0 = AB[0], AB1 = AB[1], AB2 = AB[2], CD0 = CD[0], CD1 = CD[1], CD2 = CD[2];
     constexpr int NC = ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD);
     R Gc[NC], tmp[NC];
     double f = 1.0;

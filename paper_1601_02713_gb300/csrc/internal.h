@@ -65,14 +65,24 @@ long long class_grad_flops(int cp);   // per primitive quartet of the gradient
 // ignores the choice)
 // tau_prim: primitive quartets with qp_i qp_j max|D block| below it are skipped (0: none)
 // fxs > 0: G accumulated as fixed-point integers scaled by fxs (deterministic mode, det_add)
+// df: of the FP64 part, quartets with bound < df.tau run in float-float
+// arithmetic (dfloat.cuh) where the class has a straight-line kernel
+struct DfBuild {
+    double tau;           // 0: none
+    int stage;            // 0: all launches; 1: the float-float ones; 2: the others
+    const dfloat* D;      // the density as float-floats
+    const dfloat* boys;   // the FP64 Boys table as float-floats
+};
 void launch_jk(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles,
-               const double* D, const float* Df, double* G, const double* boys, const float* boysf, double tau,
-               double fp32_tau, const double* Dsh, unsigned long long* cnt, int bs, double tau_prim, double fxs,
-               cudaStream_t st);
+               const double* D, const float* Df, const DfBuild& df, double* G, const double* boys,
+               const float* boysf, double tau, double fp32_tau, const double* Dsh, unsigned long long* cnt, int bs,
+               double tau_prim, double fxs, cudaStream_t st);
 // kernel variants generated for a class pair: the cooperative tape
 // kernel and the straight-line kernel, for the Fock build and the gradient
 bool class_pair_coop(int cp);
 bool class_pair_straight(int cp);
+bool class_pair_df(int cp);
+bool grad_pair_df(int cp);
 bool grad_pair_coop(int cp);
 bool grad_pair_straight(int cp);
 void launch_schwarz(int pair_class, const Pairs& P, const Shells& S, const int* list, int n, const double* boys,
@@ -88,11 +98,16 @@ void launch_prim_schwarz(int pair_class, const Pairs& P, const Shells& S, const 
 // (tau_prim: primitive quartets with (qg_i qp_j + qp_i qg_j) |Gamma| below it are skipped; 0 none)
 // cnt[0..1]: executed FP64 quartets and primitive quartets, cnt[2..3] FP32
 void launch_grad2e(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles,
-                   const double* D, double* grad, const double* boys, const float* boysf, double tau,
+                   const double* D, const DfBuild& df, double* grad, const double* boys, const float* boysf, double tau,
                    double fp32_tau, const double* Dsh, unsigned long long* cnt, int variant, int bs,
                    double tau_prim, double fxs, cudaStream_t st);
 void grad2e_tapes_upload();   // once per device
-void boys_table_upload(double** dev_tab, float** dev_tabf);
+void boys_table_upload(double** dev_tab, float** dev_tabf, dfloat** dev_tabd);
+// float-float copies: n values; the pairs' A - B vectors [3][npair]
+void launch_to_dfloat(const double* src, dfloat* dst, long long n, cudaStream_t st);
+// *flag = 1 if some of the n values is above lim in magnitude or not a number, else 0
+void launch_any_above(const double* v, long long n, double lim, int* flag, cudaStream_t st);
+void launch_pair_vectors(const Pairs& P, const Shells& S, dfloat* abd, cudaStream_t st);
 // FP32 copies for the mixed-precision quartets
 void launch_to_float(const double* src, float* dst, long long n, cudaStream_t st);
 

@@ -14,6 +14,8 @@
 //   V^m(0,0) = (2 pi / p) K F_m(p |PC|^2)     (and the same rule for b+1_i with PB).
 #include <math.h>
 
+#include <algorithm>
+
 #include "eri_kernels.cuh"
 #include "internal.h"
 #include "nuclear.cuh"
@@ -524,7 +526,7 @@ void boys_fill_table(double* tab)
     for (int k = 0; k < BOYS_NE; k++) tab[BOYS_EXP_OFF + k] = (double)expl(-(long double)k / BOYS_GRID);
 }
 
-void boys_table_upload(double** dev_tab, float** dev_tabf)
+void boys_table_upload(double** dev_tab, float** dev_tabf, dfloat** dev_tabd)
 {
     static double host[BOYS_TAB_DOUBLES];
     static float hostf[BOYS_TAB_FLOATS];
@@ -544,6 +546,47 @@ void boys_table_upload(double** dev_tab, float** dev_tabf)
     cudaMemcpy(*dev_tab, host, sizeof(host), cudaMemcpyHostToDevice);
     cudaMalloc(dev_tabf, sizeof(hostf));
     cudaMemcpy(*dev_tabf, hostf, sizeof(hostf), cudaMemcpyHostToDevice);
+    cudaMalloc(dev_tabd, sizeof(dfloat) * BOYS_TAB_DOUBLES);
+    launch_to_dfloat(*dev_tab, *dev_tabd, BOYS_TAB_DOUBLES, nullptr);
+    cudaStreamSynchronize(nullptr);
+}
+
+__global__ void to_dfloat_kernel(const double* src, dfloat* dst, long long n)
+{
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        dst[i] = dfloat(src[i]);
+}
+
+void launch_to_dfloat(const double* src, dfloat* dst, long long n, cudaStream_t st)
+{
+    if (n <= 0) return;
+    to_dfloat_kernel<<<(int)std::min<long long>((n + 255) / 256, 1024), 256, 0, st>>>(src, dst, n);
+}
+
+__global__ void any_above_kernel(const double* v, long long n, double lim, int* flag)
+{
+    bool any = false;
+    for (long long i = threadIdx.x; i < n; i += blockDim.x) any = any || !(fabs(v[i]) <= lim);
+    const int f = __syncthreads_or(any);
+    if (threadIdx.x == 0) *flag = f != 0;
+}
+
+void launch_any_above(const double* v, long long n, double lim, int* flag, cudaStream_t st)
+{
+    any_above_kernel<<<1, 256, 0, st>>>(v, n, lim, flag);
+}
+
+__global__ void pair_vectors_kernel(Pairs P, Shells S, dfloat* abd)
+{
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= P.n) return;
+    for (int x = 0; x < 3; x++) abd[(size_t)x * P.n + g] = dfloat(S.xyz[3 * P.sa[g] + x] - S.xyz[3 * P.sb[g] + x]);
+}
+
+void launch_pair_vectors(const Pairs& P, const Shells& S, dfloat* abd, cudaStream_t st)
+{
+    if (P.n == 0) return;
+    pair_vectors_kernel<<<(P.n + 127) / 128, 128, 0, st>>>(P, S, abd);
 }
 
 __global__ void to_float_kernel(const double* src, float* dst, long long n)

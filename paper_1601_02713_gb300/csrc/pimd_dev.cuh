@@ -9,6 +9,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "dfloat.cuh"
+
 #define PIMD_MAXPRIM 3                       // primitives per contracted shell
 #define PIMD_MAXPP (PIMD_MAXPRIM * PIMD_MAXPRIM)
 #define PIMD_LMAX 2                          // s, p, d shells
@@ -43,6 +45,7 @@ struct Shells {           // all replicas concatenated
     const int* bf;        // first basis function within the replica
     const int* atom;      // global atom index
     const int* rep;       // replica index
+    const dfloat* xyzd;   // xyz as float-floats
 };
 
 struct Pairs {
@@ -56,6 +59,8 @@ struct Pairs {
     const float* qp;      // qp[k * n + g]: Schwarz factor sqrt(max |(ij|ij)|) of primitive pair k alone
                           // (contraction coefficients included); the primitive pairs of every shell
                           // pair are stored in descending order of it
+    const dfloat* ppd;    // pp as float-floats
+    const dfloat* abd;    // [3][n] A - B of the pair's shells (centre of sa minus centre of sb)
     const float* qg;      // qg[k * n + g] = qp_k 2 sqrt(2 max(a_k, b_k)): the scale of the derivative
                           // integrals of primitive pair k (d/dA of a Gaussian of exponent a ~ sqrt(2a))
 };

@@ -45,6 +45,7 @@ struct pimd_basis {
     // flattened primitives (element-major, shell order) for the device
     std::vector<double> exps, coefs;
     std::vector<std::vector<int>> prim_off;  // per element, per shell
+    bool df_range = true;                    // exponents within the range of the float-float kernels
     long long uid = 0;                       // distinct per basis created in the process
 };
 
@@ -90,6 +91,7 @@ struct pimd_ctx {
     cudaStream_t stream = nullptr;
     double* boys = nullptr;
     float* boysf = nullptr;
+    dfloat* boysd = nullptr;
     std::map<std::string, DevBuf> bufs;
     std::string last_error;
     pimd_stats stats{};
@@ -230,7 +232,7 @@ extern "C" int pimd_ctx_create(pimd_ctx** out, int device)
         delete ctx;
         return PIMD_ECUDA;
     }
-    boys_table_upload(&ctx->boys, &ctx->boysf);
+    boys_table_upload(&ctx->boys, &ctx->boysf, &ctx->boysd);
     grad2e_tapes_upload();
     for (int i = 0; i < 8; i++) cudaEventCreate(&ctx->ev[i]);
     cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming);
@@ -260,6 +262,7 @@ extern "C" void pimd_ctx_destroy(pimd_ctx* ctx)
     }
     if (ctx->boys) cudaFree(ctx->boys);
     if (ctx->boysf) cudaFree(ctx->boysf);
+    if (ctx->boysd) cudaFree(ctx->boysd);
     for (int i = 0; i < 8; i++) cudaEventDestroy(ctx->ev[i]);
     for (int i = 0; i < pimd_ctx::kSide; i++) {
         if (ctx->side[i]) {
@@ -337,6 +340,7 @@ extern "C" int pimd_basis_create(pimd_basis** out, int nelem, const int* Z_of_el
                     return PIMD_EINVAL;
                 }
             }
+            for (int i = 0; i < d.nprim; i++) b->df_range = b->df_range && d.exps[i] > 1e-6 && d.exps[i] < 1e8;
             normalise(d);
             offs.push_back((int)b->exps.size());
             for (int i = 0; i < d.nprim; i++) {
@@ -425,6 +429,7 @@ extern "C" int pimd_last_stats(const pimd_ctx* ctx, pimd_stats* out)
 // ---------------------------------------------------------------------------
 struct Batch {
     int nrep = 0;
+    bool df_ok = false;         // float-float kernels allowed: exponents and coordinates within their range
     bool allow_odd = false;     // isolated atoms of the SAD guess (occupations set by the caller)
     std::vector<int> natom, atom0, nbf, nocc;
     std::vector<int> atom_f0;   // first function of each atom within its replica
@@ -585,7 +590,10 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
         UPLOAD("sh_src", src, d_src);
         gather_xyz(d_xyz, d_src, nsh, d_shxyz, ctx->stream);
     }
-    bt.S = Shells{d_shxyz, d_l, d_bf, d_satom, d_srep};
+    dfloat* d_shxyzd;
+    ENSURE("sh_xyzd", (size_t)nsh * 3, d_shxyzd);
+    launch_to_dfloat(d_shxyz, d_shxyzd, (long long)nsh * 3, ctx->stream);
+    bt.S = Shells{d_shxyz, d_l, d_bf, d_satom, d_srep, d_shxyzd};
 
     // replicas
     int* d_nbf;
@@ -625,7 +633,7 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
     ENSURE("npp", npair, d_npp);
     ENSURE("pp", (size_t)PP_NF * PIMD_MAXPP * npair, d_pp);
     ENSURE("Q", npair, d_Q);
-    bt.P = Pairs{npair, d_pa, d_pb, d_npp, d_pp, d_Q, nullptr, nullptr, nullptr};
+    bt.P = Pairs{npair, d_pa, d_pb, d_npp, d_pp, d_Q};
     launch_pair_data(bt.P, d_npp, d_pp, bt.S, bt.B, ctx->stream);
     ctx->stats.kernel_launches += 2;
     for (int X = 0; X < 6; X++) {
@@ -640,6 +648,11 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
         ctx->stats.kernel_launches++;
     }
     CK(cudaGetLastError());
+    int* d_far;
+    int far = 0;
+    ENSURE("far", 1, d_far);
+    launch_any_above(d_xyz, 3LL * a0, 1e4, d_far, ctx->stream);
+    CK(cudaMemcpyAsync(&far, d_far, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     std::vector<double> Q(npair);
     std::vector<int> npp(npair);
     if (npair) {
@@ -647,6 +660,7 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
         CK(cudaMemcpyAsync(npp.data(), d_npp, sizeof(int) * npair, cudaMemcpyDeviceToHost, ctx->stream));
     }
     CK(cudaStreamSynchronize(ctx->stream));
+    bt.df_ok = basis->df_range && !far;
     for (int q = 0; q < npair; q++)
         if (!isfinite(Q[q])) return set_err(ctx, PIMD_EINVAL, "non-finite integrals (check coordinates)");
     {
@@ -679,7 +693,11 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
         float *d_qp, *d_qg;
         ENSURE("qp", (size_t)PIMD_MAXPP * npair, d_qp);
         ENSURE("qg", (size_t)PIMD_MAXPP * npair, d_qg);
-        bt.P = Pairs{npair, d_pa, d_pb, d_npp, d_pp, d_Q, d_ppf, d_qp, d_qg};
+        dfloat *d_ppd, *d_abd;
+        ENSURE("ppd", (size_t)PP_NF * PIMD_MAXPP * npair, d_ppd);
+        ENSURE("abd", (size_t)3 * npair, d_abd);
+        bt.P = Pairs{npair, d_pa, d_pb, d_npp, d_pp, d_Q, d_ppf, d_qp, d_ppd, d_abd, d_qg};
+        launch_pair_vectors(bt.P, bt.S, d_abd, ctx->stream);
         launch_pair_data(bt.P, d_npp, d_pp, bt.S, bt.B, ctx->stream);
         // primitive-pair bounds, and each pair's primitives in descending order of them
         for (int X = 0; X < 6; X++) {
@@ -694,6 +712,7 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
             ctx->stats.kernel_launches++;
         }
         launch_to_float(d_pp, d_ppf, (long long)PP_NF * PIMD_MAXPP * npair, ctx->stream);
+        launch_to_dfloat(d_pp, d_ppd, (long long)PP_NF * PIMD_MAXPP * npair, ctx->stream);
     }
     // quartet tiles: for bra pair i of class X and each run of ket pairs of
     // class Y <= X with equal primitive count, the ket pairs with
@@ -899,19 +918,17 @@ static void diag_density(pimd_ctx* ctx, const Batch& bt, Mats& m, ScfPlan& p, co
     ctx->stats.kernel_launches += 2;
 }
 
-// Launch fn(cp, stream) for every class pair with tiles, the k-th on stream
-// k mod (side streams + 1) (0: the context stream), after everything already
-// queued on the context stream; the context stream then waits for all of them.
+// Launch fn(k, stream) for k = 0..n-1, the k-th on stream k mod (side streams
+// + 1) (0: the context stream), after everything already queued on the context
+// stream; the context stream then waits for all of them.
 template <class Fn>
-static int fan_out_class_pairs(pimd_ctx* ctx, const Batch& bt, Fn&& fn)
+static int fan_out(pimd_ctx* ctx, int n, Fn&& fn)
 {
     constexpr int ns = pimd_ctx::kSide + 1;
     CK(cudaEventRecord(ctx->fork_ev, ctx->stream));
     bool used[pimd_ctx::kSide] = {};
-    int k = 0;
-    for (int cp = 0; cp < n_class_pairs(); cp++) {
-        if (bt.tiles[cp].empty()) continue;
-        const int j = k++ % ns;
+    for (int k = 0; k < n; k++) {
+        const int j = k % ns;
         cudaStream_t st = ctx->stream;
         if (j > 0) {
             st = ctx->side[j - 1];
@@ -920,7 +937,7 @@ static int fan_out_class_pairs(pimd_ctx* ctx, const Batch& bt, Fn&& fn)
                 used[j - 1] = true;
             }
         }
-        fn(cp, st);
+        fn(k, st);
     }
     for (int i = 0; i < pimd_ctx::kSide; i++)
         if (used[i]) {
@@ -930,11 +947,36 @@ static int fan_out_class_pairs(pimd_ctx* ctx, const Batch& bt, Fn&& fn)
     return PIMD_OK;
 }
 
+// The launches (class pair, DfBuild stage) of a Fock build or gradient in
+// descending order of their work per quartet: the FP64 kernels of the classes
+// without a float-float one (is_df), the float-float kernels, then what is left
+// to FP64 in their classes.
+template <class IsDf>
+static std::vector<std::pair<int, int>> class_jobs(const Batch& bt, IsDf&& is_df)
+{
+    std::vector<std::pair<int, int>> jobs;
+    for (int pass = 0; pass < 3; pass++)
+        for (int cp = n_class_pairs() - 1; cp >= 0; cp--)
+            if (!bt.tiles[cp].empty() && (is_df(cp) ? pass > 0 : pass == 0)) jobs.push_back({cp, pass});
+    return jobs;
+}
+
+// The FP64 quartets whose density-weighted bound is below this run in
+// float-float arithmetic (dfloat.cuh; not for shell exponents or coordinates
+// outside its range). Their rounding error, a few 1e-14 of an integral, is then
+// below what FP64 leaves in the largest integrals: error of G against an
+// unscreened FP64 build, for 4 (H2O)8 beads / a Diels-Alder image / (H2O)16 /
+// one H2O, in units of |G|: 5.31e-13 / 2.67e-13 / 1.02e-12 / 9.55e-15 at the
+// 1e-12 integral cutoff without it and the same to three digits with it; at
+// 1e-2 H2O's is 1.26e-14. (Without any cutoff 4.1e-16 / 1.1e-15 / 3.4e-16 /
+// 5.0e-17 become 1.8e-15 / 6.5e-15 / 2.8e-15 / 3.4e-16.)
+constexpr double kDfTau = 1e-3;
+
 // G' += G'(M) over all class pairs for the replicas in the active mask, with
 // the quartets screened by Q_ab Q_cd max|M block| >= tau; those below fp32_tau
 // (if > 0) are evaluated in FP32 from Mf, an FP32 copy of M made here
 static int fock_build(pimd_ctx* ctx, Batch& bt, Mats& m, double tau, double fp32_tau, const double* M,
-                      double tau_prim, double fxs)
+                      double tau_prim, double fxs, double df_tau = kDfTau)
 {
     // deterministic mode: the build accumulates into G' as fixed-point integers
     if (fxs > 0) launch_double_to_fixed(m.G, bt.mtot, fxs, ctx->stream);
@@ -946,10 +988,24 @@ static int fock_build(pimd_ctx* ctx, Batch& bt, Mats& m, double tau, double fp32
         launch_to_float(M, Mf, bt.mtot, ctx->stream);
         ctx->stats.kernel_launches++;
     }
-    const int rc = fan_out_class_pairs(ctx, bt, [&](int cp, cudaStream_t st) {
-        launch_jk(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), M, Mf, m.G, ctx->boys, ctx->boysf,
-                  tau, fp32_tau, bt.Dsh, bt.cnt + 4 * cp, ctx->tile_w[cp], tau_prim, fxs, st);
-        ctx->stats.kernel_launches += fp32_tau > tau ? 2 : 1;
+    DfBuild df{df_tau, 0, nullptr, ctx->boysd};
+    if (bt.df_ok && df.tau > std::max(tau, fp32_tau)) {
+        dfloat* Md;
+        ENSURE("Md", bt.mtot, Md);
+        launch_to_dfloat(M, Md, bt.mtot, ctx->stream);
+        ctx->stats.kernel_launches++;
+        df.D = Md;
+    } else {
+        df.tau = 0.0;
+    }
+    const auto jobs = class_jobs(bt, [&](int cp) { return df.tau > 0.0 && class_pair_df(cp); });
+    const int rc = fan_out(ctx, (int)jobs.size(), [&](int k, cudaStream_t st) {
+        const int cp = jobs[k].first;
+        DfBuild d = df;
+        d.stage = jobs[k].second;
+        launch_jk(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), M, Mf, d, m.G, ctx->boys,
+                  ctx->boysf, tau, fp32_tau, bt.Dsh, bt.cnt + 4 * cp, ctx->tile_w[cp], tau_prim, fxs, st);
+        ctx->stats.kernel_launches += 1 + (fp32_tau > tau && d.stage != 1);
     });
     if (rc) return rc;
     if (fxs > 0) {
@@ -1062,7 +1118,7 @@ static int sad_atomic(pimd_ctx* ctx, const pimd_basis* basis, const std::vector<
         launch_delta_density(m.rm, n, m.D, m.Dp, m.dD, m.G, d_mode, st);
         // fixed-point accumulation: the cached atomic densities do not depend on
         // the order of the additions
-        if ((rc = fock_build(ctx, bt, m, 1e-12, 0.0, m.dD, 0.0, kFixG))) return rc;
+        if ((rc = fock_build(ctx, bt, m, 1e-12, 0.0, m.dD, 0.0, kFixG, 0.0))) return rc;
         launch_fock_assemble(m.rm, n, m.H, m.G, m.F, m.active, st);
         launch_copy_mats(m.rm, n, m.F, m.Fb, nullptr, st);
         if ((rc = density())) return set_err(ctx, rc, "SAD: atom without a 2p shell in the basis");
@@ -1344,6 +1400,8 @@ static int run_batch(pimd_ctx* ctx, int nrep, const int* natom_of, const int* Zc
         float* Mf;
         ENSURE("Mf", bt.mtot, Mf);   // allocated before any capture
     }
+    dfloat* Md;
+    ENSURE("Md", bt.mtot, Md);
     double* Gsum = nullptr;   // force-split mode: G' summed over the processes
     if (split) ENSURE("Gsum", bt.mtot, Gsum);
     int *d_mode, *d_slot, *d_count, *d_on;
@@ -1486,13 +1544,22 @@ static int run_batch(pimd_ctx* ctx, int nrep, const int* natom_of, const int* Zc
         }
         CK(cudaEventRecord(ctx->ev[4], ctx->stream));
         launch_shell_bounds(bt.S, bt.R, nrep, bt.maxsh, m.D, bt.Dsh, nullptr, ctx->stream);
-        const int rcg = fan_out_class_pairs(ctx, bt, [&](int cp, cudaStream_t st) {
-            launch_grad2e(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), m.D, d_grad, ctx->boys,
+        DfBuild df{bt.df_ok && kDfTau > std::max(o->schwarz_tau * 1e-2, o->fp32_tau) ? kDfTau : 0.0, 0, Md, ctx->boysd};
+        if (df.tau > 0.0) {
+            launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);
+            ctx->stats.kernel_launches++;
+        }
+        const auto jobs = class_jobs(bt, [&](int cp) { return df.tau > 0.0 && grad_pair_df(cp) && ctx->grad_var[cp] == 1; });
+        const int rcg = fan_out(ctx, (int)jobs.size(), [&](int k, cudaStream_t st) {
+            const int cp = jobs[k].first;
+            DfBuild d = df;
+            d.stage = jobs[k].second;
+            launch_grad2e(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), m.D, d, d_grad, ctx->boys,
                           ctx->boysf, o->schwarz_tau * 1e-2, o->fp32_tau, bt.Dsh, bt.cnt + 4 * 64 + 4 * cp,
                           ctx->grad_var[cp],
                           ctx->tile_w[cp] > 0 ? ctx->tile_w[cp] : 128, o->schwarz_tau * o->prim_screen,
                           fx_grad, st);
-            ctx->stats.kernel_launches += o->fp32_tau > 0 ? 2 : 1;
+            ctx->stats.kernel_launches += 1 + (o->fp32_tau > 0 && d.stage != 1);
         });
         if (rcg) return rcg;
         CK(cudaEventRecord(ctx->ev[5], ctx->stream));
@@ -1827,9 +1894,14 @@ extern "C" int pimd_autotune(pimd_ctx* ctx, int nrep, int natom, const int* Z, c
         cudaMemsetAsync(m.G, 0, sizeof(double) * bt.mtot, ctx->stream);
         launch_shell_bounds(bt.S, bt.R, bt.nrep, bt.maxsh, m.D, bt.Dsh, bt.R.active, ctx->stream);
         if (Mf) launch_to_float(m.D, Mf, bt.mtot, ctx->stream);
+        DfBuild df{bt.df_ok && kDfTau > std::max(o.schwarz_tau, o.fp32_tau) ? kDfTau : 0.0, 0, nullptr, ctx->boysd};
+        dfloat* Md;
+        if ((rc2 = dev_ensure(ctx, "Md", (size_t)bt.mtot, &Md))) break;
+        launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);
+        df.D = Md;
         rc2 = timed(ms, 4, ci, use, [&](int cp) {
             if (!bt.tiles[cp].empty())
-                launch_jk(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), m.D, Mf, m.G, ctx->boys,
+                launch_jk(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), m.D, Mf, df, m.G, ctx->boys,
                           ctx->boysf, o.schwarz_tau, o.fp32_tau, bt.Dsh, bt.cnt + 4 * cp, cand[ci],
                           o.schwarz_tau * o.prim_screen, 0.0, ctx->stream);
         });
@@ -1854,12 +1926,18 @@ extern "C" int pimd_autotune(pimd_ctx* ctx, int nrep, int natom, const int* Z, c
         if (!rc2) rc2 = dev_ensure(ctx, "tune_grad", (size_t)nrep * natom * 3, &d_g);
         if (!rc2) {
             launch_shell_bounds(bt.S, bt.R, nrep, bt.maxsh, m.D, bt.Dsh, nullptr, ctx->stream);
+            DfBuild df{bt.df_ok && kDfTau > std::max(o.schwarz_tau * 1e-2, o.fp32_tau) ? kDfTau : 0.0, 0, nullptr,
+                       ctx->boysd};
+            dfloat* Md = nullptr;
+            rc2 = dev_ensure(ctx, "Md", (size_t)bt.mtot, &Md);
+            if (!rc2) launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);
+            df.D = Md;
             for (int v = 0; v < 2 && !rc2; v++) {
                 std::vector<int> use(ncp, 0);
                 for (int cp = 0; cp < ncp; cp++)
                     use[cp] = (v == 0 ? grad_pair_coop(cp) : grad_pair_straight(cp)) && !bt.tiles[cp].empty();
                 rc2 = timed(gms, 2, v, use, [&](int cp) {
-                    launch_grad2e(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), m.D, d_g,
+                    launch_grad2e(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), m.D, df, d_g,
                                   ctx->boys, ctx->boysf, o.schwarz_tau * 1e-2, o.fp32_tau, bt.Dsh,
                                   bt.cnt + 4 * 64 + 4 * cp, v,
                                   ctx->tile_w[cp] > 0 ? ctx->tile_w[cp] : 128,
