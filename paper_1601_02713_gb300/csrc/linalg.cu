@@ -18,10 +18,14 @@ namespace pimd {
 
 namespace {
 
-// C = alpha op(A) op(B) + beta C, row-major; op(X) = X or X^T. 64x64 tiles,
-// 256 threads, 4x4 outputs per thread. grid = (tilesN, tilesM, ndesc).
-constexpr int TB = 64, TK = 16;
+// C = alpha op(A) op(B) + beta C, row-major; op(X) = X or X^T. TB x TB tiles,
+// 256 threads, (TB / 16)^2 outputs per thread. grid = (tilesN, tilesM, ndesc).
+// Bound by the FP64 pipes of the SMs that have a tile: 64 x 64 re-reads the
+// operands least, but one (H2O)8 bead (n = 192) has 9 such tiles for 152 SMs
+// and a product took 167 us; the smaller tiles spread it (launch_gemm).
+constexpr int TK = 16;
 
+template <int TB>
 __global__ void __launch_bounds__(256) gemm_kernel(const GemmDesc* __restrict__ descs, const int* active)
 {
     const GemmDesc d = descs[blockIdx.z];
@@ -30,12 +34,13 @@ __global__ void __launch_bounds__(256) gemm_kernel(const GemmDesc* __restrict__ 
     if (m0 >= d.M || n0 >= d.N) return;
     __shared__ double As[TK][TB + 1];
     __shared__ double Bs[TK][TB + 1];
+    constexpr int TM = TB / 16;
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    double acc[4][4];
+    double acc[TM][TM];
 #pragma unroll
-    for (int i = 0; i < 4; i++)
+    for (int i = 0; i < TM; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = 0.0;
+        for (int j = 0; j < TM; j++) acc[i][j] = 0.0;
     for (int k0 = 0; k0 < d.K; k0 += TK) {
         for (int e = threadIdx.x; e < TK * TB; e += 256) {
             const int kk = e / TB, mm = e % TB;
@@ -51,25 +56,25 @@ __global__ void __launch_bounds__(256) gemm_kernel(const GemmDesc* __restrict__ 
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < TK; kk++) {
-            double a[4], b[4];
+            double a[TM], b[TM];
 #pragma unroll
-            for (int i = 0; i < 4; i++) a[i] = As[kk][ty * 4 + i];
+            for (int i = 0; i < TM; i++) a[i] = As[kk][ty * TM + i];
 #pragma unroll
-            for (int j = 0; j < 4; j++) b[j] = Bs[kk][tx * 4 + j];
+            for (int j = 0; j < TM; j++) b[j] = Bs[kk][tx * TM + j];
 #pragma unroll
-            for (int i = 0; i < 4; i++)
+            for (int i = 0; i < TM; i++)
 #pragma unroll
-                for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < TM; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
-        const int m = m0 + ty * 4 + i;
+    for (int i = 0; i < TM; i++) {
+        const int m = m0 + ty * TM + i;
         if (m >= d.M) continue;
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            const int n = n0 + tx * 4 + j;
+        for (int j = 0; j < TM; j++) {
+            const int n = n0 + tx * TM + j;
             if (n >= d.N) continue;
             double* c = d.C + (size_t)m * d.ldc + n;
             *c = d.alpha * acc[i][j] + (d.beta != 0.0 ? d.beta * *c : 0.0);
@@ -99,6 +104,44 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
+// The rotation of a column pair with squared norms al, be and inner product ga:
+// false if |ga| <= tol sqrt(al be), else c, s and tg = t ga (the norms become
+// al - tg and be + tg). t solves ga t^2 + (be - al) t - ga = 0; an FP32
+// solution and one Newton step in FP64 (its derivative in FP32) give it to
+// about 1e-14, and c = 1/sqrt(1 + t^2) is formed in FP64 from that t, so the
+// rotation is orthogonal to rounding: about 25 FP64 instructions, where the
+// closed form's divisions and square roots took some 150, more than the columns
+// themselves (n = 192: 6 elements per lane). The scale 2^-e of al + be keeps
+// the FP32 numbers in range; should ga still be out of it, the closed form is
+// used.
+__device__ __forceinline__ bool jac_rotation(double al, double be, double ga, double tol, double& c, double& s,
+                                             double& tg)
+{
+    const int e = (__double2hiint(al + be) >> 20) & 0x7ff;
+    if (e >= 2046) return false;   // overflow or not a number
+    const double sc = __hiloint2double((2046 - e) << 20, 0);
+    const double a = al * sc, b = be * sc, g = ga * sc;
+    if (!(g * g > tol * tol * a * b)) return false;
+    const double d = b - a;
+    const float gf = (float)g, df = (float)d;
+    double t;
+    if (fabsf(gf) > 1e-30f) {
+        const float z = df / (2.0f * gf);
+        // |z| + sqrt(1 + z^2) = 2 |z| to FP32 from 1e9 on, where z^2 might overflow
+        const float tf = copysignf(1.0f / (fabsf(z) < 1e9f ? fabsf(z) + sqrtf(fmaf(z, z, 1.0f)) : 2.0f * fabsf(z)), z);
+        t = (double)tf;
+        const double f = fma(fma(g, t, d), t, -g);
+        t -= (double)((float)f / fmaf(2.0f * gf, tf, df));
+    } else {
+        const double zeta = d / (2.0 * g);
+        t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+    }
+    c = rsqrt_r(fma(t, t, 1.0));
+    s = c * t;
+    tg = t * ga;
+    return true;
+}
+
 // PER = column elements held per lane (n <= 32 PER): the kernel is FP64-bound,
 // so PER is the smallest instantiated length that fits the batch's largest
 // matrix (padding lanes would be FP64 work on zeros).
@@ -109,6 +152,10 @@ __device__ __forceinline__ double warp_sum(double v)
 // per round. Every CTA computes the shift and the column norms of the
 // eigenvalue step itself (O(n^2), small); the rotation flag of a sweep is
 // or-ed into CTA 0's shared memory (distributed shared memory).
+// The squared column norms are kept in nrm (the eigenvalues' place until the
+// end): formed from the columns at the start of every sweep and updated by the
+// rotations, so a pair needs one inner product instead of three.
+// 32 matrices of n = 192 (an SCF step's diagonalisation): 28.4 -> 17.0 ms.
 // notconv (may be NULL): notconv[r] = 1 when matrix r is still rotating after
 // JAC_MAXSWEEP sweeps (its eigenpairs are then not converged)
 template <int CS>
@@ -136,6 +183,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const RepMat* __res
     double* G = work + rm.off;     // column-major: G[col * n + row]
     double* v = V + rm.off;
     double* ev = evals + (size_t)r * ldE;
+    double* nrm = ev;
     __shared__ double s_red[JAC_THREADS / 32];
     __shared__ double s_shift;
     __shared__ int s_rot[3];       // CTA 0's copy: rotation flags of sweeps s mod 3
@@ -174,6 +222,18 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const RepMat* __res
         // sweep - 2, and every CTA has passed a barrier of sweep - 1 since
         if (cr == 0 && threadIdx.x == 0) s_rot[(sweep + 1) % 3] = 0;
         int rotated = 0;
+        for (int j = warp * CS + cr; j < n; j += nw * CS) {
+            double nn = 0.0;
+#pragma unroll
+            for (int k = 0; k < PER; k++) {
+                const int i = lane + 32 * k;
+                const double x = i < n ? G[(size_t)j * n + i] : 0.0;
+                nn = fma(x, x, nn);
+            }
+            nn = warp_sum(nn);
+            if (lane == 0) nrm[j] = nn;
+        }
+        jac_cluster_sync<CS>();
         for (int rd = 0; rd < M - 1; rd++) {
             for (int k = warp * CS + cr; k < M / 2; k += nw * CS) {
                 int p, q;
@@ -195,21 +255,18 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const RepMat* __res
                     x[k] = i < n ? gp[i] : 0.0;
                     y[k] = i < n ? gq[i] : 0.0;
                 }
-                double al = 0.0, be = 0.0, ga = 0.0;
+                const double al = nrm[p], be = nrm[q];
+                double ga = 0.0;
 #pragma unroll
-                for (int k = 0; k < PER; k++) {
-                    al = fma(x[k], x[k], al);
-                    be = fma(y[k], y[k], be);
-                    ga = fma(x[k], y[k], ga);
-                }
-                al = warp_sum(al);
-                be = warp_sum(be);
+                for (int k = 0; k < PER; k++) ga = fma(x[k], y[k], ga);
                 ga = warp_sum(ga);
-                if (fabs(ga) > tol * sqrt(al * be) && ga != 0.0) {
+                double c, s, tg;
+                if (jac_rotation(al, be, ga, tol, c, s, tg)) {
                     rotated = 1;
-                    const double zeta = (be - al) / (2.0 * ga);
-                    const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-                    const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
+                    if (lane == 0) {
+                        nrm[p] = al - tg;
+                        nrm[q] = be + tg;
+                    }
 #pragma unroll
                     for (int k = 0; k < PER; k++) {
                         const int i = lane + 32 * k;
@@ -676,8 +733,15 @@ void add_mats(const RepMat* rm, int nrep, const double* A, const double* B, doub
 void launch_gemm(const GemmDesc* d_desc, int ndesc, int maxM, int maxN, const int* active, cudaStream_t st)
 {
     if (ndesc == 0 || maxM == 0 || maxN == 0) return;
-    dim3 grid((maxN + TB - 1) / TB, (maxM + TB - 1) / TB, ndesc);
-    gemm_kernel<<<grid, 256, 0, st>>>(d_desc, active);
+    // the largest tile that gives every SM one
+    auto blocks = [&](int tb) { return (long long)((maxN + tb - 1) / tb) * ((maxM + tb - 1) / tb) * ndesc; };
+    auto grid = [&](int tb) { return dim3((maxN + tb - 1) / tb, (maxM + tb - 1) / tb, ndesc); };
+    if (blocks(64) >= 152)
+        gemm_kernel<64><<<grid(64), 256, 0, st>>>(d_desc, active);
+    else if (blocks(32) >= 152)
+        gemm_kernel<32><<<grid(32), 256, 0, st>>>(d_desc, active);
+    else
+        gemm_kernel<16><<<grid(16), 256, 0, st>>>(d_desc, active);
 }
 
 void launch_jacobi(const RepMat* d_rm, int nrep, const double* A, double* V, double* evals, int ldE, double* work,
