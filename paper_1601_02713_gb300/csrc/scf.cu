@@ -725,6 +725,15 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
     bt.nquart_rep.assign(nrep, 0);
     bt.vrr_flops = 0.0;
     bt.eris = 0.0;
+    // first pair of each run, and the end of the last, of every (replica, class)
+    // group: found once, not once per bra pair (finding them for each bra walked
+    // all the group's pairs and took 100 of the 146 ms of the set-up at (H2O)16)
+    std::vector<std::vector<int>> runs(bt.grp0.size() - 1);
+    for (size_t g = 0; g < runs.size(); g++) {
+        for (int q = bt.grp0[g]; q < bt.grp0[g + 1]; q++)
+            if (q == bt.grp0[g] || bt.npp[q] != bt.npp[q - 1]) runs[g].push_back(q);
+        runs[g].push_back(bt.grp0[g + 1]);
+    }
     for (int X = 0; X < 6; X++)
         for (int Y = 0; Y <= X; Y++) {
             const int cp = class_pair_index(X, Y);
@@ -732,13 +741,12 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
             auto& tl = bt.tiles[cp];
             for (int r = 0; r < nrep; r++) {
                 const int b0 = bt.grp0[r * 6 + X], b1 = bt.grp0[r * 6 + X + 1];
-                const int k0 = bt.grp0[r * 6 + Y], k1 = bt.grp0[r * 6 + Y + 1];
+                const std::vector<int>& run = runs[(size_t)r * 6 + Y];
                 for (int i = b0; i < b1; i++) {
                     if (Q[i] <= 0.0) continue;
                     const double thr = tau / Q[i];
-                    for (int s0 = k0; s0 < k1;) {
-                        int s1 = s0;
-                        while (s1 < k1 && bt.npp[s1] == bt.npp[s0]) s1++;
+                    for (size_t u = 0; u + 1 < run.size(); u++) {
+                        const int s0 = run[u], s1 = run[u + 1];
                         // first index in [s0, s1) with Q < thr (Q descending within the run)
                         int lo = s0, hi = s1;
                         while (lo < hi) {
@@ -754,7 +762,6 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
                             bt.nquart_rep[r] += nqi;
                             for (int c = s0; c < kend; c += tw) tl.push_back(Tile{i, c, std::min(c + tw, kend), r});
                         }
-                        s0 = s1;
                     }
                 }
             }
