@@ -121,8 +121,9 @@ def generate_sources():
     coop_e = {s[0]: s[7] for s in stats}
     coop_g = {s[0]: s[8] for s in stats}
     straight_e = {s[0]: s[9] for s in stats}
-    df_e = {s[0]: s[10] for s in stats}
-    df_g = {s[0]: s[11] for s in stats}
+    df_e = straight_e   # every straight-line class has a float-float Fock kernel
+    df_g = {s[0]: s[10] for s in stats}
+    df_all = {s[0]: s[11] for s in stats}
     classes = g.classes()
     names = [g.cls_name(c) for c in classes]
     tus = []
@@ -160,15 +161,16 @@ def generate_sources():
         if straight_e[nm]:
             e += ["    const int b = bs > 0 ? bs : 128;",
                   "    const dim3 grid(ntiles, jk_blocks_per_tile(ntiles));"]
-            if df_e[nm]:
-                e += ["    const double top = df.tau > split ? df.tau : split;",
-                      "    if (top > split && df.stage != 2)",
-                      f"        jk_kernel<Cls_{nm}, dfloat><<<grid, b, 0, st>>>(P, S, R, tiles, df.D, G, df.boys, split, top,",
-                      "                                                        Dsh, cnt, tp, fxs);"]
-            else:
-                e += ["    const double top = split;"]
-            e += ["    if (df.stage == 1) return;",
-                  f"    jk_kernel<Cls_{nm}, double><<<grid, b, 0, st>>>(P, S, R, tiles, D, G, boys, top, 1e300, Dsh, cnt,",
+            top = "1e300" if df_all[nm] else "df.tau"
+            e += [f"    const double top = df.tau > split ? {top} : split;",
+                  "    if (top > split && df.stage != 2)",
+                  f"        jk_kernel<Cls_{nm}, dfloat><<<grid, b, 0, st>>>(P, S, R, tiles,",
+                  f"                                                        tail_density<Cls_{nm}>(D, df.D), G,",
+                  "                                                        df.boys, split, top, Dsh, cnt, DF_TAU_PRIM * tp,",
+                  "                                                        fxs);",
+                  "    if (df.stage == 1) return;",
+                  "    if (top < 1e300)",
+                  f"        jk_kernel<Cls_{nm}, double><<<grid, b, 0, st>>>(P, S, R, tiles, D, G, boys, top, 1e300, Dsh, cnt,",
                   "                                                      tp, fxs);",
                   "    if (fp32_tau > tau)",
                   f"        jk_kernel<Cls_{nm}, float><<<ntiles, b, 0, st>>>(P, S, R, tiles, Df, G, boysf, tau, fp32_tau, Dsh,",
@@ -291,7 +293,8 @@ def generate_sources():
              "double tau, double fp32_tau, const double* Dsh, unsigned long long* cnt, int bs, double tau_prim, "
              "double fxs, cudaStream_t st)")
     d.append("{ jk_tab[cp](P, S, R, tiles, ntiles, D, Df, df, G, boys, boysf, tau, fp32_tau, Dsh, cnt, bs, tau_prim, fxs, st); }")
-    for fn, tab in (("class_pair_coop", coop_e), ("class_pair_straight", straight_e), ("grad_pair_coop", coop_g), ("class_pair_df", df_e), ("grad_pair_df", df_g),
+    for fn, tab in (("class_pair_coop", coop_e), ("class_pair_straight", straight_e), ("grad_pair_coop", coop_g),
+                    ("class_pair_df", df_e), ("class_pair_df_all", df_all), ("grad_pair_df", df_g),
                     ("grad_pair_straight", {nm: not heavy[nm] for nm in names})):
         d.append(f"bool {fn}(int cp)")
         d.append("{")

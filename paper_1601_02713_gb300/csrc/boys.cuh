@@ -177,15 +177,16 @@ __device__ __forceinline__ void boys_eval(dfloat T, const dfloat* __restrict__ t
     if (T.h < (float)BOYS_TMAX) {
         const float kf = rintf(T.h * (float)BOYS_GRID);
         const int k = (int)kf;
-        // T_k and T.h are multiples of ulp(T.h) at most 1/32 apart: exact
-        const dfloat x(__fsub_rn(kf * (1.0f / BOYS_GRID), T.h), -T.l);
+        // T_k and T.h are multiples of ulp(T.h) at most 1/32 apart: exact. The low
+        // part of T need not be small against the difference, hence the full sum.
+        const dfloat x = two_sum(__fsub_rn(kf * (1.0f / BOYS_GRID), T.h), -T.l);
         const dfloat* t = tab + ((size_t)k * BOYS_MT + L) * BOYS_NTAYLOR;
         float r = ldg(t + 7).h;
         r = fmaf(r, x.h, ldg(t + 6).h);
         r = fmaf(r, x.h, ldg(t + 5).h);
         r = fmaf(r, x.h, ldg(t + 4).h);
         const dfloat t3 = ldg(t + 3);
-        dfloat f(t3.h, fmaf(r, x.h, t3.l));
+        dfloat f = fast_two_sum(t3.h, fmaf(r, x.h, t3.l));
         f = boys_horner(f, x, ldg(t + 2));
         f = boys_horner(f, x, ldg(t + 1));
         f = boys_horner(f, x, ldg(t));
@@ -195,7 +196,7 @@ __device__ __forceinline__ void boys_eval(dfloat T, const dfloat* __restrict__ t
             e = fmaf(e, x.h, 1.0f / 120.0f);
             e = fmaf(e, x.h, 1.0f / 24.0f);
             constexpr dfloat c3(1.0 / 6.0);
-            dfloat ex(c3.h, fmaf(e, x.h, c3.l));
+            dfloat ex = fast_two_sum(c3.h, fmaf(e, x.h, c3.l));
             ex = boys_horner(ex, x, dfloat(0.5f, 0.0f));
             ex = boys_horner(ex, x, dfloat(1.0f, 0.0f));
             ex = boys_horner(ex, x, dfloat(1.0f, 0.0f));

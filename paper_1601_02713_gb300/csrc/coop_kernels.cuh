@@ -160,9 +160,9 @@ __device__ __forceinline__ void coop_prim(const Pairs& P, int ab, int cd, int k,
                                           const R* __restrict__ boys, R* g)
 {
     const int i = k % npp_ab, j = k / npp_ab;
-    R bra[PP_NF], ket[PP_NF];
-    load_ppn(P, ab, i, bra, PP_NF);
-    load_ppn(P, cd, j, ket, PP_NF);
+    R bra[PP_EB + 1], ket[PP_EB + 1];
+    load_ppn(P, ab, i, bra, PP_EB + 1);
+    load_ppn(P, cd, j, ket, PP_EB + 1);
     PrimQ<R> q;
     prim_quartet<R>(bra, ket, q);
     for (int x = 0; x < 3; x++) {

@@ -90,4 +90,40 @@ __device__ __forceinline__ dfloat rsqrt_r(dfloat x)
     return dfloat(y, __fmul_rn(y, __fmaf_rn(__fmul_rn(0.375f, e), e, __fmul_rn(0.5f, e))));
 }
 
+// Two float-floats side by side: every operation is the packed (f32x2) form of
+// the scalar one, which issues one instruction for both lanes.
+struct dfloat2 {
+    float2 h, l;
+    __device__ dfloat2() {}
+    __device__ dfloat2(float2 a, float2 b) : h(a), l(b) {}
+    __device__ dfloat2(dfloat a, dfloat b) : h(make_float2(a.h, b.h)), l(make_float2(a.l, b.l)) {}
+    __device__ dfloat lane0() const { return dfloat(h.x, l.x); }
+    __device__ dfloat lane1() const { return dfloat(h.y, l.y); }
+};
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ dfloat2 exchange(dfloat2 a)
+{
+    return dfloat2(make_float2(a.h.y, a.h.x), make_float2(a.l.y, a.l.x));
+}
+__device__ __forceinline__ dfloat2 two_sum(float2 a, float2 b)
+{
+    const float2 s = __fadd2_rn(a, b), t = __fadd2_rn(s, neg2(a));
+    return dfloat2(s, __fadd2_rn(__fadd2_rn(a, neg2(__fadd2_rn(s, neg2(t)))), __fadd2_rn(b, neg2(t))));
+}
+__device__ __forceinline__ dfloat2 operator*(dfloat2 a, dfloat2 b)
+{
+    const float2 p = __fmul2_rn(a.h, b.h);
+    return dfloat2(p, __ffma2_rn(a.l, b.h, __ffma2_rn(a.h, b.l, __ffma2_rn(a.h, b.h, neg2(p)))));
+}
+__device__ __forceinline__ dfloat2 operator+(dfloat2 a, dfloat2 b)
+{
+    const dfloat2 s = two_sum(a.h, b.h);
+    return dfloat2(s.h, __fadd2_rn(s.l, __fadd2_rn(a.l, b.l)));
+}
+__device__ __forceinline__ dfloat2 fma(dfloat2 a, dfloat2 b, dfloat2 c)
+{
+    const dfloat2 p = a * b, s = two_sum(c.h, p.h);
+    return dfloat2(s.h, __fadd2_rn(__fadd2_rn(s.l, c.l), p.l));
+}
+
 }  // namespace pimd

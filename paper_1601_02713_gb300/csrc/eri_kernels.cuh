@@ -26,6 +26,19 @@
 
 namespace pimd {
 
+// Float-float Fock kernels, by the operations of the class's recursion: above
+// the first, the packed recursion (two nodes to an instruction; (dp|ps) 17.7 ->
+// 15.3 ms, (dp|dp) 62.5 -> 36.9 for 8 (H2O)8 beads, but (pp|ps), below it, 12.3
+// -> 13.0: the packed form costs registers and its gain is code size); above
+// the second, the horizontal recursion, transform and J/K contraction in FP64
+// ((dp|ps) 15.3 -> 13.3 ms, (dp|ds) 19.3 -> 16.7): the FP64 pipe is idle, and
+// their code leaves the instruction caches to the primitive loop.
+constexpr int DF_PACKED_MIN_FLOPS = 300, DF_TAIL64_MIN_FLOPS = 500;
+// their primitive cutoff as a fraction of the FP64 kernels': what it keeps more
+// outweighs the float-float rounding in the error of the Fock matrix (kDfTau
+// has the figures), for 1% of the time
+constexpr double DF_TAU_PRIM = 0.8;
+
 constexpr double kSqrt3 = 1.7320508075688772935;
 
 // in[N0][ncart(L)][N2] -> out[N0][nsph(L)][N2]; spherical d order m = -2..2:
@@ -143,15 +156,39 @@ __device__ __forceinline__ void prim_quartet(const R* bra, const R* ket, PrimQ<R
     g.theta = bra[PP_K] * ket[PP_K] * rs;
 }
 
-// The same from float-float pair data. P - Q is formed as AC + (P - A) -
-// (Q - C) with AC the vector between the bra's and the ket's first centre: the
-// differences are exact zeros where the centres coincide (the largest
-// integrals), where the difference of two coordinates would leave 2^-48 of
-// the coordinates themselves. aq = AC - (Q - C), formed once per ket primitive.
-__device__ __forceinline__ void prim_quartet(const dfloat* bra, const dfloat* ket, const dfloat* aq,
-                                             PrimQ<dfloat>& g)
+// How the float-float kernels form P - Q of a quartet: as (P - X) - (Q - Y) +
+// (X - Y) with X the bra centre A or B and Y the ket centre C or D, on the same
+// atom where the quartet has such a pair. The product centres of two tight
+// primitives can then be as close as they are (the integral varies over
+// 1/sqrt(rho)), where a difference of coordinates, or of a centre other than the
+// near one, would leave 2^-48 of a bond length or of the molecule's size.
+struct DfCentres {
+    int bra, ket;     // first of the three fields P - X: PP_PAX or PP_PBX
+    dfloat XY[3];
+    __device__ __forceinline__ DfCentres(const Shells& S, int sa, int sb, int sc, int sd)
+    {
+        const int a = S.atom[sa], b = S.atom[sb], c = S.atom[sc], d = S.atom[sd];
+        bra = a == c || a == d || (b != c && b != d) ? PP_PAX : PP_PBX;
+        ket = (bra == PP_PAX ? a : b) == d && (bra == PP_PAX ? a : b) != c ? PP_PBX : PP_PAX;
+        const int x = bra == PP_PAX ? sa : sb, y = ket == PP_PAX ? sc : sd;
+#pragma unroll
+        for (int k = 0; k < 3; k++) XY[k] = ldg(S.xyzd + 3 * x + k) - ldg(S.xyzd + 3 * y + k);
+    }
+    // X - Y - (Q - Y) of ket primitive j of pair cd
+    __device__ __forceinline__ void ket_part(const Pairs& P, int cd, int j, dfloat aq[3]) const
+    {
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+            aq[k] = XY[k] - ldg(P.ppd + ((size_t)(ket + k) * PIMD_MAXPP + j) * P.n + cd);
+    }
+};
+
+// The same from float-float pair data: bra primitive i of sbra, aq from
+// DfCentres::ket_part.
+__device__ __forceinline__ void prim_quartet(const dfloat (*sbra)[PIMD_MAXPP], int i, const DfCentres& ctr,
+                                             const dfloat* ket, const dfloat* aq, PrimQ<dfloat>& g)
 {
-    const dfloat p = bra[PP_P], q = ket[PP_P];
+    const dfloat p = sbra[PP_P][i], q = ket[PP_P];
     const dfloat rs = rsqrt_r(p + q);
     const dfloat ipq = rs * rs;
     const dfloat qi = q * ipq, pi = p * ipq;
@@ -159,20 +196,24 @@ __device__ __forceinline__ void prim_quartet(const dfloat* bra, const dfloat* ke
     dfloat PQ[3];
 #pragma unroll
     for (int x = 0; x < 3; x++) {
-        g.PA[x] = bra[PP_PAX + x];
+        g.PA[x] = sbra[PP_PAX + x][i];
         g.QC[x] = ket[PP_PAX + x];
-        PQ[x] = aq[x] + g.PA[x];
+        PQ[x] = aq[x] + sbra[ctr.bra + x][i];
         g.WP[x] = -(qi * PQ[x]);
         g.WQ[x] = pi * PQ[x];
     }
     g.T = renorm(rho * fma(PQ[0], PQ[0], fma(PQ[1], PQ[1], PQ[2] * PQ[2])));
-    g.o2p = bra[PP_O2P];
-    g.o2pr = rho * bra[PP_O2PP];
+    g.o2p = sbra[PP_O2P][i];
+    g.o2pr = rho * sbra[PP_O2PP][i];
     g.o2q = ket[PP_O2P];
     g.o2qr = rho * ket[PP_O2PP];
     g.o2pq = scale2(ipq, 0.5f);
-    g.theta = bra[PP_K] * ket[PP_K] * rs;
+    g.theta = sbra[PP_K][i] * ket[PP_K] * rs;
 }
+
+// rows of a kernel's shared bra data
+template <typename R>
+constexpr int bra_rows(int n) { return std::is_same<R, dfloat>::value ? (int)PP_NF : n; }
 
 __device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
@@ -403,16 +444,36 @@ __device__ __forceinline__ int stair_total(const float* sqp, int nbra, const Pai
 // contracted accumulators are summed over them before the horizontal
 // recursion. Every lane of the warp calls this (total = 0: no quartet; cd then
 // any pair); kmax: the longest sequence of the warp.
+// Float-float classes: which ones use the packed recursion, and which hand the
+// contracted accumulators to FP64 for the horizontal recursion, the spherical
+// transform and the J/K contraction (Tail: the type of those).
 template <class C, typename R>
+struct DfClass {
+    static constexpr bool df = std::is_same<R, dfloat>::value;
+    static constexpr bool packed = df && C::VRR_FLOPS > DF_PACKED_MIN_FLOPS;
+    typedef typename std::conditional<df && (C::VRR_FLOPS > DF_TAIL64_MIN_FLOPS), double, R>::type Tail;
+};
+template <typename R>
+__device__ __forceinline__ R to_tail(R v, R) { return v; }
+__device__ __forceinline__ double to_tail(dfloat v, double) { return (double)v; }
+
+template <class C, typename R, typename T>
 __device__ __forceinline__ void quartet_cart(const R (*sbra)[PIMD_MAXPP], const float* sqp, int nbra, const Pairs& P,
-                                             int cd, const R AB[3], const R CD[3], const R AC[3],
+                                             int cd, const T AB[3], const T CD[3], const DfCentres* ctr,
                                              const R* __restrict__ boys, float qthr, int total, int kmax, int S,
-                                             int sub, R* cart)
+                                             int sub, T* cart)
 {
-    constexpr bool DF = std::is_same<R, dfloat>::value;
+    constexpr bool DF = std::is_same<R, dfloat>::value, PACKED = DfClass<C, R>::packed;
+    // (the float-float recursion is packed, two nodes to an operation)
     R acc[C::NE * C::NF];
+    dfloat2 acc2[PACKED ? C::N2 : 1];
+    if constexpr (PACKED) {
 #pragma unroll
-    for (int i = 0; i < C::NE * C::NF; i++) acc[i] = R(0);
+        for (int i = 0; i < C::N2; i++) acc2[i] = dfloat2(make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f));
+    } else {
+#pragma unroll
+        for (int i = 0; i < C::NE * C::NF; i++) acc[i] = R(0);
+    }
     // position `pos` of the sequence = bra primitive i of ket primitive j,
     // whose row is w long
     int i = sub, j = 0, jl = -1;
@@ -428,29 +489,47 @@ __device__ __forceinline__ void quartet_cart(const R (*sbra)[PIMD_MAXPP], const 
             if (j != jl) {
                 load_ppn(P, cd, j, ket, PP_NERI);
                 jl = j;
-                if constexpr (DF)
-#pragma unroll
-                    for (int x = 0; x < 3; x++) aq[x] = AC[x] - ket[PP_PAX + x];
+                if constexpr (DF) ctr->ket_part(P, cd, j, aq);
             }
-            R bra[PP_NERI];
-#pragma unroll
-            for (int f = 0; f < PP_NERI; f++) bra[f] = sbra[f][i];
             PrimQ<R> g;
-            if constexpr (DF)
-                prim_quartet(bra, ket, aq, g);
-            else
+            if constexpr (DF) {
+                prim_quartet(sbra, i, *ctr, ket, aq, g);
+            } else {
+                R bra[PP_NERI];
+#pragma unroll
+                for (int f = 0; f < PP_NERI; f++) bra[f] = sbra[f][i];
                 prim_quartet<R>(bra, ket, g);
+            }
             R F[C::L + 1];
             boys_eval<C::L>(g.T, boys, g.theta, F);
-            C::template vrr<R>(F, g.PA[0], g.PA[1], g.PA[2], g.WP[0], g.WP[1], g.WP[2], g.QC[0], g.QC[1], g.QC[2],
-                               g.WQ[0], g.WQ[1], g.WQ[2], g.o2p, g.o2pr, g.o2q, g.o2qr, g.o2pq, acc);
+            if constexpr (PACKED) {
+                // what a long recursion reads many times, with normalised low parts
+#pragma unroll
+                for (int m = 0; m <= C::L; m++) F[m] = renorm(F[m]);
+#pragma unroll
+                for (int x = 0; x < 3; x++) {
+                    g.WP[x] = renorm(g.WP[x]);
+                    g.WQ[x] = renorm(g.WQ[x]);
+                }
+                g.o2pr = renorm(g.o2pr);
+                g.o2qr = renorm(g.o2qr);
+                g.o2pq = renorm(g.o2pq);
+                C::vrr2(F, g, acc2);
+            }
+            else
+                C::template vrr<R>(F, g.PA[0], g.PA[1], g.PA[2], g.WP[0], g.WP[1], g.WP[2], g.QC[0], g.QC[1], g.QC[2],
+                                   g.WQ[0], g.WQ[1], g.WQ[2], g.o2p, g.o2pr, g.o2q, g.o2qr, g.o2pq, acc);
             i += S;
         }
     }
+    if constexpr (PACKED) C::vrr2_unpack(acc2, acc);
     for (int o = 1; o < S; o <<= 1)
 #pragma unroll
         for (int e = 0; e < C::NE * C::NF; e++) acc[e] += shfl_xor(acc[e], o);
-    if (sub == 0) C::template hrr<R>(acc, AB[0], AB[1], AB[2], CD[0], CD[1], CD[2], cart);
+    T acct[C::NE * C::NF];
+#pragma unroll
+    for (int e = 0; e < C::NE * C::NF; e++) acct[e] = to_tail(acc[e], T());
+    if (sub == 0) C::template hrr<T>(acct, AB[0], AB[1], AB[2], CD[0], CD[1], CD[2], cart);
 }
 
 // Blocks per tile of the straight-line kernels (gridDim.y): a block takes every
@@ -458,9 +537,6 @@ __device__ __forceinline__ void quartet_cart(const R (*sbra)[PIMD_MAXPP], const 
 // lanes per quartet, so a small batch's primitive loops are spread over the
 // chip instead of running 81 recursions deep on a few warps. Batches with two
 // blocks of 128 threads per SM already fill the register files.
-// With the float-float kernels: the Fock build of one water molecule 18.8 ->
-// 6.3 ms, the forces of 4 minimal-basis dimers 37.3 -> 12.5 ms, of one (H2O)8
-// bead 1196 -> 843 ms.
 inline int jk_blocks_per_tile(int ntiles)
 {
     const int want = 4 * 152;
@@ -472,17 +548,20 @@ inline int jk_blocks_per_tile(int ntiles)
 // fixed-point integers (det_add).
 template <class C, typename R>
 __global__ void __launch_bounds__(128) jk_kernel(Pairs P, Shells S_, Reps R_, const Tile* __restrict__ tiles,
-                                                 const R* __restrict__ Dall, double* __restrict__ Gall,
+                                                 const typename DfClass<C, R>::Tail* __restrict__ Dall,
+                                                 double* __restrict__ Gall,
                                                  const R* __restrict__ boys, double tau_lo, double tau_hi,
                                                  const double* __restrict__ Dsh, unsigned long long* __restrict__ cnt,
                                                  double tau_prim, double fxs)
 {
-    __shared__ R sbra[PP_NERI][PIMD_MAXPP];
+    typedef typename DfClass<C, R>::Tail T;
+    constexpr int ROWS = bra_rows<R>(PP_NERI);
+    __shared__ R sbra[ROWS][PIMD_MAXPP];
     __shared__ float sqp[PIMD_MAXPP];
     const Tile t = tiles[blockIdx.x];
     if (!R_.active[t.rep]) return;
     const int ab = t.ab;
-    for (int e = threadIdx.x; e < PP_NERI * PIMD_MAXPP; e += blockDim.x) {
+    for (int e = threadIdx.x; e < ROWS * PIMD_MAXPP; e += blockDim.x) {
         const int f = e / PIMD_MAXPP, k = e % PIMD_MAXPP;
         sbra[f][k] = pp_base(P, R())[((size_t)f * PIMD_MAXPP + k) * P.n + ab];
     }
@@ -553,24 +632,28 @@ __global__ void __launch_bounds__(128) jk_kernel(Pairs P, Shells S_, Reps R_, co
     // sums over lanes (the block's warps share the bra pair)
     if (__all_sync(0xffffffffu, !work)) return;
     constexpr int NCART = ncart(C::LA) * ncart(C::LB) * ncart(C::LC) * ncart(C::LD);
-    R cart[NCART], tmp[NCART];
+    T cart[NCART], tmp[NCART];
     const int total = work ? stair_total(sqp, nbra, P, cd, qthr) : 0;
     const int kmax = __reduce_max_sync(0xffffffffu, (unsigned)total);
-    R AB[3], CD[3], AC[3];
+    T AB[3], CD[3];
     if (work) {
 #pragma unroll
         for (int x = 0; x < 3; x++) {
-            if constexpr (std::is_same<R, dfloat>::value) {
+            if constexpr (std::is_same<T, dfloat>::value) {
                 AB[x] = ldg(P.abd + (size_t)x * P.n + ab);
                 CD[x] = ldg(P.abd + (size_t)x * P.n + cd);
-                AC[x] = ldg(S_.xyzd + 3 * sa + x) - ldg(S_.xyzd + 3 * sc + x);
             } else {
-                AB[x] = R(S_.xyz[3 * sa + x] - S_.xyz[3 * sb + x]);
-                CD[x] = R(S_.xyz[3 * sc + x] - S_.xyz[3 * sd + x]);
+                AB[x] = T(S_.xyz[3 * sa + x] - S_.xyz[3 * sb + x]);
+                CD[x] = T(S_.xyz[3 * sc + x] - S_.xyz[3 * sd + x]);
             }
         }
     }
-    quartet_cart<C, R>(sbra, sqp, nbra, P, cd, AB, CD, AC, boys, qthr, total, kmax, S, sub, cart);
+    if constexpr (DfClass<C, R>::df) {
+        const DfCentres ctr(S_, sa, sb, work ? sc : sa, work ? sd : sb);
+        quartet_cart<C, R, T>(sbra, sqp, nbra, P, cd, AB, CD, &ctr, boys, qthr, total, kmax, S, sub, cart);
+    } else {
+        quartet_cart<C, R, T>(sbra, sqp, nbra, P, cd, AB, CD, nullptr, boys, qthr, total, kmax, S, sub, cart);
+    }
     work = work && sub == 0;
     double f = 0.0;
     if (work) {
@@ -589,10 +672,10 @@ __global__ void __launch_bounds__(128) jk_kernel(Pairs P, Shells S_, Reps R_, co
     }
     const int N = R_.nbf[r];
     const size_t off = R_.moff[r];
-    bra_coulomb_warp<C::LA, C::LB, C::LC, C::LD, R>(cart, f, work, S_.bf[P.sa[ab]], S_.bf[P.sb[ab]], S_.bf[sc],
+    bra_coulomb_warp<C::LA, C::LB, C::LC, C::LD, T>(cart, f, work, S_.bf[P.sa[ab]], S_.bf[P.sb[ab]], S_.bf[sc],
                                                      S_.bf[sd], N, Dall + off, Gall + off, fxs);
     if (work)
-        scatter_jk<C::LA, C::LB, C::LC, C::LD, R>(cart, f, S_.bf[sa], S_.bf[sb], S_.bf[sc], S_.bf[sd], N, Dall + off,
+        scatter_jk<C::LA, C::LB, C::LC, C::LD, T>(cart, f, S_.bf[sa], S_.bf[sb], S_.bf[sc], S_.bf[sd], N, Dall + off,
                                                   Gall + off, fxs, false);
 }
 
@@ -627,6 +710,16 @@ __device__ __forceinline__ void pair_block(const Pairs& P, const double* pp, int
     double tmp[NCART];
     C::template hrr<double>(acc, A[0] - B[0], A[1] - B[1], A[2] - B[2], A[0] - B[0], A[1] - B[1], A[2] - B[2], cart);
     cart_to_sph4<C::LA, C::LB, C::LC, C::LD>(cart, tmp);
+}
+
+// the density the float-float kernel of class C contracts with
+template <class C>
+static const typename DfClass<C, dfloat>::Tail* tail_density(const double* D, const dfloat* Dd)
+{
+    if constexpr (std::is_same<typename DfClass<C, dfloat>::Tail, double>::value)
+        return D;
+    else
+        return Dd;
 }
 
 // Schwarz factors: Q_ab = sqrt(max over functions of (mn|mn)), one block per

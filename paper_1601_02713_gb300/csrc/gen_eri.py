@@ -147,6 +147,152 @@ class VRRGen:
         return f"fma({a1}, {t1}, {inner})", fl + 2
 
 
+class PackedVRRGen:
+    """The same recursion for the float-float kernels, two nodes at a time.
+    Exchanging the x and y axes maps the recursion onto itself, so a node and
+    its mirror image (e and f with x and y exchanged) are the two lanes of one
+    packed operation (f32x2), with coefficients (PA_x, PA_y) and so on: the
+    generated code is 1.5 to 1.8 times shorter. The node computed in lane 0 has
+    more x than y in f, or equal in f and more or equal in e; its recursion
+    then steps along x or z only. Nodes that are their own image fill both
+    lanes. An operand whose lanes are the wrong way round is exchanged once."""
+
+    def __init__(self):
+        self.names = {}
+        self.exchanged = {}
+        self.nodes = []      # (name, key)
+        self.lines = []
+        self.uses = {}
+        self.used_f = set()
+        self.used_c = set()
+
+    @staticmethod
+    def mirror(key):
+        e, f, m = key
+        return (e[1], e[0], e[2]), (f[1], f[0], f[2]), m
+
+    @staticmethod
+    def is_lane0(key):
+        for v in (key[1], key[0]):
+            if v[0] != v[1]:
+                return v[0] > v[1]
+        return True
+
+    @staticmethod
+    def step(key):
+        """(kind, direction, operands [(coefficient, k, key)]) of a lane-0 node"""
+        e, f, m = key
+        ket = sum(f) > 0
+        i = pick_dir(f if ket else e)
+        assert i != 1
+        down = (lambda k: (e, sub(f, i, k))) if ket else (lambda k: (sub(e, i, k), f))
+        top = (f if ket else e)[i] - 1
+        c1, c2, c3, c4 = ("QC", "WQ", "o2q", "no2qr") if ket else ("PA", "WP", "o2p", "no2pr")
+        e1, f1 = down(1)
+        ops = [(c1 + ("01" if i == 0 else "2"), 1, (e1, f1, m)), (c2 + ("01" if i == 0 else "2"), 1, (e1, f1, m + 1))]
+        if top > 0:
+            e2, f2 = down(2)
+            ops += [(c3, top, (e2, f2, m)), (c4, top, (e2, f2, m + 1))]
+        if ket and e[i] > 0:
+            ops.append(("o2pq", e[i], (sub(e, i), f1, m + 1)))
+        return ops
+
+    def visit(self, key):
+        """Collect the nodes a key needs, operands first."""
+        if not self.is_lane0(key):
+            key = self.mirror(key)
+        if sum(key[0]) == 0 and sum(key[1]) == 0:
+            self.used_f.add(key[2])
+            return
+        if key in self.names:
+            return
+        self.names[key] = None
+        ops = self.step(key)
+        for _, _, k in ops:
+            self.visit(k)
+            k0 = k if self.is_lane0(k) else self.mirror(k)
+            self.uses[k0] = self.uses.get(k0, 0) + 1
+        self.names[key] = f"v{len(self.nodes)}"
+        self.nodes.append((key, ops))
+
+    def operand(self, key):
+        if sum(key[0]) == 0 and sum(key[1]) == 0:
+            return f"F{key[2]}"
+        if self.is_lane0(key):
+            return self.names[key]
+        key = self.mirror(key)
+        if key not in self.exchanged:
+            self.exchanged[key] = f"x{self.names[key][1:]}"
+            self.lines.append(f"const dfloat2 {self.exchanged[key]} = exchange({self.names[key]});")
+        return self.exchanged[key]
+
+    def emit(self, key, ops, addend):
+        inner = addend
+        for c, k, src in reversed(ops):
+            if k > 1:
+                self.used_c.add((c, k))
+                c = f"{c}_{k}"
+            x = self.operand(src)
+            inner = f"fma({c}, {x}, {inner})" if inner else f"{c} * {x}"
+        return inner
+
+
+def gen_vrr_packed(name, acc_sets):
+    """Packed counterpart of gen_vrr: accumulates into dfloat2 arrays, one per
+    set (`name`), whose two lanes a second function (`name`_unpack) writes to
+    the scalar accumulators of gen_vrr. Returns (code, {set: packed length})."""
+    g = PackedVRRGen()
+    slots = {}     # set -> {lane-0 key: packed index}
+    unpack = []
+    for acc, elo, ehi, flo, fhi, w in acc_sets:
+        es, fs = level_range(elo, ehi), level_range(flo, fhi)
+        sl = slots.setdefault(acc, {})
+        for ie, e in enumerate(es):
+            for jf, f in enumerate(fs):
+                key = (e, f, 0)
+                lane = 0 if g.is_lane0(key) else 1
+                k0 = key if lane == 0 else g.mirror(key)
+                g.visit(k0)
+                idx = sl.setdefault(k0, len(sl))
+                unpack.append(f"{acc}[{ie * len(fs) + jf}] = {acc}2[{idx}].lane{lane}();")
+    weight = {a[0]: a[5] for a in acc_sets}
+    ntarget = {}
+    for sl in slots.values():
+        for k in sl:
+            ntarget[k] = ntarget.get(k, 0) + 1
+    fold = {k: f"{acc}2[{i}]" for acc, sl in slots.items() for k, i in sl.items()
+            if weight[acc] is None and ntarget[k] == 1 and g.uses.get(k, 0) == 0 and k in g.names}
+    for key, ops in g.nodes:
+        dst = fold.get(key)
+        ex = g.emit(key, ops, dst)
+        g.lines.append(f"{dst} = {ex};" if dst else f"const dfloat2 {g.names[key]} = {ex};")
+    for acc, sl in slots.items():
+        for k, i in sl.items():
+            if k in fold:
+                continue
+            v, w = g.operand(k), weight[acc]
+            g.lines.append(f"{acc}2[{i}] = " + (f"fma({w}, {v}, {acc}2[{i}]);" if w else f"{acc}2[{i}] + {v};"))
+    accs = list(slots)
+    ws = [weight[a] for a in accs if weight[a]]
+    args = ", ".join([f"dfloat2* __restrict__ {a}2" for a in accs] + [f"dfloat2 {w}" for w in ws])
+    head = [f"static __device__ __forceinline__ void {name}(const dfloat* __restrict__ Fm, const PrimQ<dfloat>& g, {args})",
+            "{"]
+    for m in sorted(g.used_f):
+        head.append(f"    const dfloat2 F{m}(Fm[{m}], Fm[{m}]);")
+    for v in ("PA", "WP", "QC", "WQ"):
+        head.append(f"    const dfloat2 {v}01(g.{v}[0], g.{v}[1]), {v}2(g.{v}[2], g.{v}[2]);")
+    base = {"o2p": "g.o2p", "no2pr": "-g.o2pr", "o2q": "g.o2q", "no2qr": "-g.o2qr", "o2pq": "g.o2pq"}
+    for c, ex in base.items():
+        head.append(f"    const dfloat2 {c}({ex}, {ex});")
+    for c, k in sorted(g.used_c):
+        ex = f"dfloat({k}) * ({base[c]})"
+        head.append(f"    const dfloat {c}_{k}s = {ex};\n    const dfloat2 {c}_{k}({c}_{k}s, {c}_{k}s);")
+    un = [f"static __device__ __forceinline__ void {name}_unpack("
+          + ", ".join([f"const dfloat2* {a}2" for a in accs] + [f"dfloat* {a}" for a in accs]) + ")", "{"]
+    code = head + ["    " + x for x in g.lines] + ["}"] + un + ["    " + x for x in unpack] + ["}"]
+    return "\n".join(code) + "\n", {a: len(sl) for a, sl in slots.items()}
+
+
 def level_range(lo, hi):
     out = []
     for l in range(max(lo, 0), hi + 1):
@@ -529,17 +675,17 @@ def encode_hrr(op):
 COOP_ENERGY_MIN_VRR = 2000
 STRAIGHT_ENERGY_MAX_VRR = 2000
 COOP_GRAD_MIN_VRR = 400
-# float-float Fock kernel (dfloat.cuh): up to this many operations per
-# primitive quartet. A multiply-add is 12 FP32 instructions, and above this the
-# recursion's code (tens of kilobytes) no longer stays in the instruction
-# caches: 8 (H2O)8 beads, one build, FP64 -> float-float: (ps|ss) 36.7 -> 5.2 ms,
-# (pp|ps) 51.6 -> 12.3, (dp|ps) 41.5 -> 17.7, (dp|ds), the largest in, 32.7 ->
-# 23.8; (dp|pp), the smallest out, 51.7 -> 61.3, (dp|dp) 39.3 -> 62.5.
-DF_MAX_FLOPS = 1600
-# the gradient's recursion runs to order L + 1 into four accumulator sets, so its
-# code and registers reach the limit sooner: one bead, FP64 -> float-float:
-# (ps|ss) 8.5 -> 3.0 ms, (ps|ps) 13.6 -> 4.9, (dp|ss), the largest in, 5.3 ->
-# 4.3; (ds|ps), the smallest out, 11.6 -> 11.7, (pp|ps) 24.1 -> 87.4.
+# Fock classes above this many operations per primitive quartet run all their
+# FP64 quartets in float-float arithmetic: a launch for their few largest ones
+# cost as much as a tenth of the class (FP64 (dd|dp) quartets above 1e-2 of 4
+# (H2O)8 beads: 18 ms beside 16 ms for the rest in float-float).
+DF_ALL_MIN_FLOPS = 1000
+# float-float gradient kernel: up to this many operations per primitive quartet.
+# The gradient's recursion runs to order L + 1 into four accumulator sets, and
+# beyond this its code and registers outgrow the instruction caches and the
+# register file: one bead, FP64 -> float-float: (ps|ss) 8.5 -> 3.0 ms, (ps|ps)
+# 13.6 -> 4.9, (dp|ss), the largest in, 5.3 -> 4.3; (ds|ps), the smallest out,
+# 11.6 -> 11.7, (pp|ps) 24.1 -> 87.4.
 DF_GRAD_MAX_FLOPS = 900
 
 
@@ -832,11 +978,13 @@ def generate(outdir):
         parts = [f"// Generated by gen_eri.py for class ({nm[:2]}|{nm[2:]}).\n#pragma once\n\n"]
         code, nl, nfl = gen_vrr("vrr", L, [("acc", la, la + lb, lc, lc + ld, None)])
         hcode, nh = gen_hrr("hrr", la, lb, lc, ld, la, la + lb, lc, lc + ld)
-        parts.append(f"struct Cls_{nm} {{\n  static constexpr int LA={la}, LB={lb}, LC={lc}, LD={ld}, L={L}, "
-                     f"NE={n_range(la, la + lb)}, NF={n_range(lc, lc + ld)}, VRR_FLOPS={nfl};\n")
+        pcode, npk = gen_vrr_packed("vrr2", [("acc", la, la + lb, lc, lc + ld, None)])
+        parts.append(f"namespace pimd {{\n\nstruct Cls_{nm} {{\n  static constexpr int LA={la}, LB={lb}, LC={lc}, LD={ld}, L={L}, "
+                     f"NE={n_range(la, la + lb)}, NF={n_range(lc, lc + ld)}, VRR_FLOPS={nfl}, N2={npk['acc']};\n")
         parts.append(code)
+        parts.append(pcode)
         parts.append(hcode)
-        parts.append("};\n")
+        parts.append("};\n\n}  // namespace pimd\n")
         write_if_changed(os.path.join(outdir, f"eri_{nm}.cuh"), "".join(parts))
         coop_e = nl > COOP_ENERGY_MIN_VRR
         straight_e = nl <= STRAIGHT_ENERGY_MAX_VRR
@@ -865,8 +1013,8 @@ def generate(outdir):
         if coop_g:
             hdr, _ = coop_header(nm, True, gen_coop(c, True))
             write_if_changed(os.path.join(outdir, f"coopg_{nm}.cuh"), hdr)
-        stats.append((nm, nl, nfl, nh, gnl, gnfl, heavy, coop_e, coop_g, straight_e, straight_e and nfl <= DF_MAX_FLOPS,
-                      not heavy and gnfl <= DF_GRAD_MAX_FLOPS))
+        stats.append((nm, nl, nfl, nh, gnl, gnfl, heavy, coop_e, coop_g, straight_e,
+                      not heavy and gnfl <= DF_GRAD_MAX_FLOPS, straight_e and nfl > DF_ALL_MIN_FLOPS))
     return stats
 
 

@@ -162,11 +162,12 @@ __global__ void __launch_bounds__(128) grad2e_kernel(Pairs P, Shells S, Reps Rp,
                                                      double fxs)
 {
     constexpr int LA = G::LA, LB = G::LB, LC = G::LC, LD = G::LD;
-    __shared__ R sbra[PP_NF][PIMD_MAXPP];
+    constexpr int ROWS = bra_rows<R>(PP_EB + 1);
+    __shared__ R sbra[ROWS][PIMD_MAXPP];
     __shared__ float sqp[PIMD_MAXPP], sqg[PIMD_MAXPP];
     const Tile t = tiles[blockIdx.x];
     const int ab = t.ab;
-    for (int e = threadIdx.x; e < PP_NF * PIMD_MAXPP; e += blockDim.x) {
+    for (int e = threadIdx.x; e < ROWS * PIMD_MAXPP; e += blockDim.x) {
         const int f = e / PIMD_MAXPP, k = e % PIMD_MAXPP;
         sbra[f][k] = pp_base(P, R())[((size_t)f * PIMD_MAXPP + k) * P.n + ab];
     }
@@ -257,18 +258,18 @@ __global__ void __launch_bounds__(128) grad2e_kernel(Pairs P, Shells S, Reps Rp,
     }
     constexpr bool DF = std::is_same<R, dfloat>::value;
     const int sc = work ? P.sa[cd] : sa, sd = work ? P.sb[cd] : sb;
-    R AB[3], CD[3], AC[3];
+    R AB[3], CD[3];
 #pragma unroll
     for (int x = 0; x < 3; x++) {
         if constexpr (DF) {
             AB[x] = ldg(P.abd + (size_t)x * P.n + ab);
             CD[x] = ldg(P.abd + (size_t)x * P.n + (work ? cd : ab));
-            AC[x] = ldg(S.xyzd + 3 * sa + x) - ldg(S.xyzd + 3 * sc + x);
         } else {
             AB[x] = R(S.xyz[3 * sa + x] - S.xyz[3 * sb + x]);
             CD[x] = R(S.xyz[3 * sc + x] - S.xyz[3 * sd + x]);
         }
     }
+    const DfCentres ctr(S, sa, sb, sc, sd);
     R accU[G::N_accU], accA[G::N_accA], accB[G::N_accB], accC[G::N_accC];
     for (int i = 0; i < G::N_accU; i++) accU[i] = R(0);
     for (int i = 0; i < G::N_accA; i++) accA[i] = R(0);
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(128) grad2e_kernel(Pairs P, Shells S, Reps Rp,
         qpj = __ldg(P.qp + cd);
         qgj = __ldg(P.qg + cd);
     }
-    R ket[PP_NF], aq[3];
+    R ket[PP_EB + 1], aq[3];
     for (int k = 0; k < kmax; k += lanes) {
         if (k + sub < total) {
             // advance to this lane's next surviving primitive quartet (one exists: k + sub < total)
@@ -295,20 +296,19 @@ __global__ void __launch_bounds__(128) grad2e_kernel(Pairs P, Shells S, Reps Rp,
             }
             skip = lanes;   // the one evaluated now is the first passed over
             if (j != jl) {
-                load_ppn(P, cd, j, ket, PP_NF);
+                load_ppn(P, cd, j, ket, PP_EB + 1);
                 jl = j;
-                if constexpr (DF)
-#pragma unroll
-                    for (int x = 0; x < 3; x++) aq[x] = AC[x] - ket[PP_PAX + x];
+                if constexpr (DF) ctr.ket_part(P, cd, j, aq);
             }
-            R bra[PP_NERI];
-#pragma unroll
-            for (int f = 0; f < PP_NERI; f++) bra[f] = sbra[f][i];
             PrimQ<R> g;
-            if constexpr (DF)
-                prim_quartet(bra, ket, aq, g);
-            else
+            if constexpr (DF) {
+                prim_quartet(sbra, i, ctr, ket, aq, g);
+            } else {
+                R bra[PP_NERI];
+#pragma unroll
+                for (int f = 0; f < PP_NERI; f++) bra[f] = sbra[f][i];
                 prim_quartet<R>(bra, ket, g);
+            }
             R F[G::L + 1];
             boys_eval<G::L>(g.T, boys, g.theta, F);
             G::template vrr<R>(F, g.PA[0], g.PA[1], g.PA[2], g.WP[0], g.WP[1], g.WP[2], g.QC[0], g.QC[1], g.QC[2],

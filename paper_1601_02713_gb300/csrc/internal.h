@@ -82,6 +82,7 @@ void launch_jk(int cp, const Pairs& P, const Shells& S, const Reps& R, const Til
 bool class_pair_coop(int cp);
 bool class_pair_straight(int cp);
 bool class_pair_df(int cp);
+bool class_pair_df_all(int cp);   // every FP64 quartet of the class runs in float-float arithmetic
 bool grad_pair_df(int cp);
 bool grad_pair_coop(int cp);
 bool grad_pair_straight(int cp);

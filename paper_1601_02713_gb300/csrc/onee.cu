@@ -126,7 +126,7 @@ __global__ void pair_data_kernel(Pairs P, int* npp, double* pp, Shells S, BasisP
             const double Px = (ea * A[0] + eb * Bc[0]) * ip, Py = (ea * A[1] + eb * Bc[1]) * ip,
                          Pz = (ea * A[2] + eb * Bc[2]) * ip;
             const double vals[PP_NF] = {p,  Px, Py, Pz, c0 * kij, Px - A[0], Py - A[1], Pz - A[2],
-                                        0.5 * ip, 0.5 * ip * ip, ea, eb};
+                                        0.5 * ip, 0.5 * ip * ip, ea, eb, Px - Bc[0], Py - Bc[1], Pz - Bc[2]};
             for (int f = 0; f < PP_NF; f++) pp[((size_t)f * PIMD_MAXPP + k) * P.n + g] = vals[f];
             k++;
         }

@@ -35,6 +35,7 @@ enum PPField {
     PP_O2P,               // 1 / (2p)
     PP_O2PP,              // 1 / (2p^2)
     PP_EA, PP_EB,         // exponents a, b (gradient weights)
+    PP_PBX, PP_PBY, PP_PBZ,  // P - B (float-float kernels)
     PP_NF
 };
 constexpr int PP_NERI = PP_EA;

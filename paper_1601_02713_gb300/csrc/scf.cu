@@ -970,14 +970,16 @@ static std::vector<std::pair<int, int>> class_jobs(const Batch& bt, IsDf&& is_df
 
 // The FP64 quartets whose density-weighted bound is below this run in
 // float-float arithmetic (dfloat.cuh; not for shell exponents or coordinates
-// outside its range). Their rounding error, a few 1e-14 of an integral, is then
-// below what FP64 leaves in the largest integrals: error of G against an
-// unscreened FP64 build, for 4 (H2O)8 beads / a Diels-Alder image / (H2O)16 /
-// one H2O, in units of |G|: 5.31e-13 / 2.67e-13 / 1.02e-12 / 9.55e-15 at the
-// 1e-12 integral cutoff without it and the same to three digits with it; at
-// 1e-2 H2O's is 1.26e-14. (Without any cutoff 4.1e-16 / 1.1e-15 / 3.4e-16 /
-// 5.0e-17 become 1.8e-15 / 6.5e-15 / 2.8e-15 / 3.4e-16.)
-constexpr double kDfTau = 1e-3;
+// outside its range), in the classes with long recursions all of them
+// (class_pair_df_all; their integrals are not the largest). The rounding error
+// of a few 1e-14 of an integral is then of the order of what FP64 leaves in the
+// largest integrals, and below the integral cutoffs' error. Error of the Fock
+// matrix against an unscreened FP64 build in units of its norm, all in FP64 ->
+// with this: 4 (H2O)8 beads 5.31e-13 -> 5.28e-13, a Diels-Alder image 2.67e-13 ->
+// 2.58e-13, (H2O)16 1.02e-12 -> 1.02e-12, one H2O 9.55e-15 -> 9.43e-15 (without
+// any cutoff 4e-16 / 4e-16 / 1e-15 / 9e-17 -> 1.6e-14 / 2.1e-14 / 1.2e-14 /
+// 1.2e-15; DF_TAU_PRIM makes up for that).
+constexpr double kDfTau = 1e-2;
 
 // G' += G'(M) over all class pairs for the replicas in the active mask, with
 // the quartets screened by Q_ab Q_cd max|M block| >= tau; those below fp32_tau
@@ -1005,7 +1007,9 @@ static int fock_build(pimd_ctx* ctx, Batch& bt, Mats& m, double tau, double fp32
     } else {
         df.tau = 0.0;
     }
-    const auto jobs = class_jobs(bt, [&](int cp) { return df.tau > 0.0 && class_pair_df(cp); });
+    // (a class with nothing left to FP64 is one launch, or two with FP32 quartets)
+    const auto jobs = class_jobs(
+        bt, [&](int cp) { return df.tau > 0.0 && class_pair_df(cp) && (!class_pair_df_all(cp) || fp32_tau > tau); });
     const int rc = fan_out(ctx, (int)jobs.size(), [&](int k, cudaStream_t st) {
         const int cp = jobs[k].first;
         DfBuild d = df;
