@@ -96,6 +96,10 @@ constexpr int JAC_THREADS = 512;
 constexpr int JAC_PER = 24;   // largest column length per lane: n <= 768
 constexpr int JAC_MAXSWEEP = 60;
 constexpr int JAC_CLUSTER = 8;   // CTAs (SMs) per matrix of 128 or more rows
+// up to this many matrices take twice as many (a cluster of 16 is beyond the
+// portable size; one fits each of the 8 graphics-processing clusters): the 19
+// diagonalisations of one (H2O)8 bead's SCF 98 -> 61 ms
+constexpr int JAC_FEW = 8;
 
 __device__ __forceinline__ double warp_sum(double v)
 {
@@ -312,26 +316,36 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const RepMat* __res
     if constexpr (CS > 1) cg::this_cluster().sync();
 }
 
+template <int PER, int CS>
+static void jacobi_cluster(int nmat, cudaStream_t st, size_t sm, const RepMat* rm, const double* A, double* V,
+                           double* evals, int ldE, double* work, const int* active, int shift, int* notconv)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nmat * CS);
+    cfg.blockDim = dim3(JAC_THREADS);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CS;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (CS > 8) cudaFuncSetAttribute(jacobi_kernel<PER, CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaLaunchKernelEx(&cfg, jacobi_kernel<PER, CS>, rm, A, V, evals, ldE, work, active, shift, notconv);
+}
+
 template <int PER>
 static void jacobi_launch(int nmat, cudaStream_t st, size_t sm, const RepMat* rm, const double* A, double* V,
                           double* evals, int ldE, double* work, const int* active, int shift, int* notconv)
 {
-    // matrices of 128 or more rows: a cluster of JAC_CLUSTER CTAs (SMs) each
-    if (PER >= 4) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(nmat * JAC_CLUSTER);
-        cfg.blockDim = dim3(JAC_THREADS);
-        cfg.dynamicSmemBytes = sm;
-        cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = JAC_CLUSTER;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        cudaLaunchKernelEx(&cfg, jacobi_kernel<PER, JAC_CLUSTER>, rm, A, V, evals, ldE, work, active, shift,
-                           notconv);
+    // matrices of 128 or more rows: a cluster of CTAs (SMs) each
+    if constexpr (PER >= 4) {
+        if (nmat <= JAC_FEW)
+            jacobi_cluster<PER, 2 * JAC_CLUSTER>(nmat, st, sm, rm, A, V, evals, ldE, work, active, shift, notconv);
+        else
+            jacobi_cluster<PER, JAC_CLUSTER>(nmat, st, sm, rm, A, V, evals, ldE, work, active, shift, notconv);
     } else {
         jacobi_kernel<PER, 1><<<nmat, JAC_THREADS, sm, st>>>(rm, A, V, evals, ldE, work, active, shift, notconv);
     }

@@ -107,8 +107,10 @@ struct pimd_ctx {
     // the class-pair launches of a Fock build (and of the gradient) are
     // spread over the context stream and these side streams (fork/join by
     // events, also inside a captured graph), so that one launch's last wave
-    // overlaps the next launches instead of leaving SMs idle
-    static constexpr int kSide = 3;
+    // overlaps the next launches instead of leaving SMs idle; small batches
+    // leave room for many of them (one (H2O)8 bead's Fock builds, 16 of up to 36
+    // launches: 404 ms with 3 side streams, 386 with 11)
+    static constexpr int kSide = 11;
     cudaStream_t side[kSide] = {};
     cudaEvent_t fork_ev = nullptr, join_ev[kSide] = {};
     int nsm = 152;
