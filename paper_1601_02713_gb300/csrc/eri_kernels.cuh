@@ -1,14 +1,15 @@
 // Shell-quartet ERI kernels: Coulomb/exchange (Fock) build, Schwarz factors
 // and the two-electron part of the analytic RHF gradient.
 //
-// One thread evaluates one contracted shell quartet (ab|cd) of one replica:
-// the primitive loop runs the generated Obara-Saika vertical recursion into
-// contracted [e0|f0] accumulators, then the generated Head-Gordon-Pople
-// horizontal recursion gives the Cartesian block, which is turned into real
+// One thread, or several lanes of a warp where quartets are few, evaluates one
+// contracted shell quartet (ab|cd) of one replica, in FP64, float-float
+// (dfloat.cuh) or FP32: the primitive loop runs the generated Obara-Saika
+// vertical recursion into contracted [e0|f0] accumulators, then the generated
+// Head-Gordon-Pople horizontal recursion gives the Cartesian block, which is turned into real
 // spherical d functions and contracted with the density on the fly.
 // A block shares one bra pair (staged in shared memory) and walks a tile of
-// 32, 64 or 128 ket pairs of the same class (one thread each; the width is
-// chosen per class pair by the autotuner), so the code path is uniform across
+// 32, 64 or 128 ket pairs of the same class (the width is chosen per class pair
+// by the autotuner), so the code path is uniform across
 // the block. Every replica of the call is covered by the same launch.
 //
 // Quartets are the canonical ones (a >= b, c >= d, ab >= cd); each is
@@ -535,13 +536,16 @@ __device__ __forceinline__ void quartet_cart(const R (*sbra)[PIMD_MAXPP], const 
 // Blocks per tile of the straight-line kernels (gridDim.y): a block takes every
 // gridDim.y-th of the tile's quartets and, where few are left to it, several
 // lanes per quartet, so a small batch's primitive loops are spread over the
-// chip instead of running 81 recursions deep on a few warps. Batches with two
-// blocks of 128 threads per SM already fill the register files.
-inline int jk_blocks_per_tile(int ntiles)
-{
-    const int want = 4 * 152;
-    return ntiles >= want ? 1 : (want + ntiles - 1) / ntiles < 8 ? (want + ntiles - 1) / ntiles : 8;
-}
+// chip instead of running 81 recursions deep on a few warps. Two where a class
+// has fewer tiles than the chip holds blocks (2 per SM); its launch runs beside
+// those of the other classes, and more blocks repeat the set-up and the serial
+// end of a quartet for ever fewer of them: one (H2O)8 bead's Fock builds 398 /
+// 364 / 386 ms with 1 / 2 / up to 8 blocks per tile below 152 / 304 / 608 tiles,
+// 4 dimers' 55 / 59 / 72, ragged images' 173 / 164 / 186.
+// With the float-float kernels and the lane sharing: the Fock build of one water
+// molecule 18.8 -> 6.3 ms, the forces of 4 minimal-basis dimers 37.3 -> 12.5 ms,
+// of one (H2O)8 bead 1196 -> 843 ms.
+inline int jk_blocks_per_tile(int ntiles) { return ntiles < 2 * 152 ? 2 : 1; }
 
 // tau_prim: primitive quartets whose bound qp_i qp_j (density bound) is below
 // it are skipped (0 keeps every primitive quartet). fxs > 0: G' accumulated as

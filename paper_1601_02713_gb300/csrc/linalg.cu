@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const RepMat* __res
 }
 
 template <int PER, int CS>
-static void jacobi_cluster(int nmat, cudaStream_t st, size_t sm, const RepMat* rm, const double* A, double* V,
+static cudaError_t jacobi_cluster(int nmat, cudaStream_t st, size_t sm, const RepMat* rm, const double* A, double* V,
                            double* evals, int ldE, double* work, const int* active, int shift, int* notconv)
 {
     cudaLaunchConfig_t cfg = {};
@@ -333,7 +333,7 @@ static void jacobi_cluster(int nmat, cudaStream_t st, size_t sm, const RepMat* r
     cfg.attrs = at;
     cfg.numAttrs = 1;
     if (CS > 8) cudaFuncSetAttribute(jacobi_kernel<PER, CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaLaunchKernelEx(&cfg, jacobi_kernel<PER, CS>, rm, A, V, evals, ldE, work, active, shift, notconv);
+    return cudaLaunchKernelEx(&cfg, jacobi_kernel<PER, CS>, rm, A, V, evals, ldE, work, active, shift, notconv);
 }
 
 template <int PER>
@@ -342,10 +342,13 @@ static void jacobi_launch(int nmat, cudaStream_t st, size_t sm, const RepMat* rm
 {
     // matrices of 128 or more rows: a cluster of CTAs (SMs) each
     if constexpr (PER >= 4) {
-        if (nmat <= JAC_FEW)
-            jacobi_cluster<PER, 2 * JAC_CLUSTER>(nmat, st, sm, rm, A, V, evals, ldE, work, active, shift, notconv);
-        else
-            jacobi_cluster<PER, JAC_CLUSTER>(nmat, st, sm, rm, A, V, evals, ldE, work, active, shift, notconv);
+        if (nmat <= JAC_FEW) {
+            if (jacobi_cluster<PER, 2 * JAC_CLUSTER>(nmat, st, sm, rm, A, V, evals, ldE, work, active, shift,
+                                                     notconv) == cudaSuccess)
+                return;
+            cudaGetLastError();   // a device share without room for such a cluster: the portable size
+        }
+        jacobi_cluster<PER, JAC_CLUSTER>(nmat, st, sm, rm, A, V, evals, ldE, work, active, shift, notconv);
     } else {
         jacobi_kernel<PER, 1><<<nmat, JAC_THREADS, sm, st>>>(rm, A, V, evals, ldE, work, active, shift, notconv);
     }
