@@ -57,7 +57,9 @@ typedef struct {
     int max_iter;         /* 64 */
     int diis_size;        /* 8 (Pulay subspace, 2..16) */
     double schwarz_tau;   /* 1e-12: quartets with Q_ab Q_cd below it are skipped (Sec. 3.1) */
-    double fp32_tau;      /* 0: all quartets in FP64; > schwarz_tau: quartets whose bound
+    double fp32_tau;      /* 0: no FP32 quartets (all in FP64, or as float-floats, pairs of FP32
+                             numbers, where that leaves the results no further from exact);
+                             > schwarz_tau: quartets whose bound
                              Q_ab Q_cd max|D block| is below it (D: the density increment of an
                              incremental build) are evaluated in FP32 and accumulated in FP64 */
     int guess;            /* 0 core Hamiltonian, 1 previous MOs of the same replica index (Sec. 2:
@@ -117,7 +119,7 @@ typedef struct {
     double final_dE;      /* last |E_k - E_{k-1}| */
     double final_error;   /* last max |X^T (FDS - SDF) X| */
     long long nquartets;  /* screened shell quartets per Fock build */
-    long long nq_fp64;    /* shell quartets of the replica executed in FP64, all Fock builds of the call */
+    long long nq_fp64;    /* shell quartets of the replica executed in FP64 (or float-float), all Fock builds of the call */
     long long nq_fp32;    /* ... and in FP32 (mixed mode: bound below fp32_tau) */
 } pimd_info;
 
