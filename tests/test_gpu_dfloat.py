@@ -31,11 +31,15 @@ def _density(N, nrep, seed):
     return D + D.transpose(0, 2, 1)
 
 
-def _gpu(ctx, B, Z, Xs, D):
+def _gpu_tau(ctx, B, Z, Xs, D, tau):
     Dt = torch.tensor(D, device="cuda")
     G = torch.zeros_like(Dt)
-    native.pimd_fock_dev(ctx, B, Z, Xs, Dt, G, 1e-12)
+    native.pimd_fock_dev(ctx, B, Z, Xs, Dt, G, tau)
     return G.cpu().numpy()
+
+
+def _gpu(ctx, B, Z, Xs, D):
+    return _gpu_tau(ctx, B, Z, Xs, D, 1e-12)
 
 
 def _check(bas, Z, Xs, D, G, tol=TOL):
@@ -101,25 +105,24 @@ def test_far_coordinates(ctx):
     assert not np.array_equal(G1, G0)
 
 
-@pytest.mark.parametrize("tau", [0.0, 1e-15])
-def test_tight_cutoffs_keep_fp64(ctx, tau):
-    """A cutoff below the default asks for less than the float-float rounding
-    (some 1e-14 of the Fock matrix): the build is then the FP64 one, forced here
-    by an element outside the float-float range that the molecule does not hold.
-    The two differ by the order of the atomic additions alone: some 1e2 terms of
-    2^-53 of an element's largest, with random signs 1e-15."""
+@pytest.mark.parametrize("tau,fp64", [(0.0, True), (1e-15, True), (1e-12, False)])
+def test_tight_cutoffs_keep_fp64(ctx, tau, fp64):
+    """A cutoff below the default asks for less than the float-float rounding:
+    the build then takes the FP64 path, launch for launch the one that an element
+    outside the float-float range forces (the molecule does not hold it)."""
     bas = inputs.basis_set("split_spd")
     wide = dict(bas)
     wide[2] = [inputs.Shell(0, [1e9], [1.0])]
-    Z, Xs = inputs.beads(*inputs.water_cluster_geometry(4, 2), 1, 5).stacked()
+    Z, Xs = inputs.beads(*inputs.water_cluster_geometry(1, 2), 1, 5).stacked()
     B = native.Basis(bas)
-    D = torch.tensor(_density(B.nbf(Z), 1, 6), device="cuda")
-    G = []
-    for b in (B, native.Basis(wide)):
-        g = torch.zeros_like(D)
-        native.pimd_fock_dev(ctx, b, Z, Xs, D, g, tau)
-        G.append(g.cpu().numpy())
-    assert np.linalg.norm(G[0] - G[1]) < 1e-15 * np.linalg.norm(G[1])
+    D = _density(B.nbf(Z), 1, 6)
+
+    def launches(b):
+        n0 = native.pimd_last_stats(ctx)["kernel_launches"]
+        _gpu_tau(ctx, b, Z, Xs, D, tau)
+        return native.pimd_last_stats(ctx)["kernel_launches"] - n0
+
+    assert (launches(B) == launches(native.Basis(wide))) == fp64
 
 
 @pytest.mark.parametrize("n,nmat", [(1, 3), (2, 1), (31, 2), (64, 5), (65, 1), (127, 2), (129, 1), (193, 1)])
