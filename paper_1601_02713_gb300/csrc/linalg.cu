@@ -260,6 +260,9 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const RepMat* __res
                     y[k] = i < n ? gq[i] : 0.0;
                 }
                 const double al = nrm[p], be = nrm[q];
+                // every lane's read of the norms comes before lane 0's update
+                // of them below (the shuffles of warp_sum order no memory)
+                __syncwarp();
                 double ga = 0.0;
 #pragma unroll
                 for (int k = 0; k < PER; k++) ga = fma(x[k], y[k], ga);
