@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(256) gemm_kernel(const GemmDesc* __restrict__ 
 constexpr int JAC_THREADS = 512;
 constexpr int JAC_PER = 24;   // largest column length per lane: n <= 768
 constexpr int JAC_MAXSWEEP = 60;
-constexpr int JAC_CLUSTER = 8;   // CTAs (SMs) per matrix of 128 or more rows
+constexpr int JAC_CLUSTER = 8;   // CTAs (SMs) per matrix of a batch with more than 64 rows
 // up to this many matrices take twice as many (a cluster of 16 is beyond the
 // portable size; one fits each of the 8 graphics-processing clusters): the 19
 // diagonalisations of one (H2O)8 bead's SCF 98 -> 61 ms
@@ -319,39 +319,63 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const RepMat* __res
     if constexpr (CS > 1) cg::this_cluster().sync();
 }
 
-template <int PER, int CS>
-static cudaError_t jacobi_cluster(int nmat, cudaStream_t st, size_t sm, const RepMat* rm, const double* A, double* V,
-                           double* evals, int ldE, double* work, const int* active, int shift, int* notconv)
+// launch configuration of clusters of cs CTAs, one cluster per matrix
+static cudaLaunchConfig_t jacobi_config(int nmat, int cs, size_t sm, cudaStream_t st, cudaLaunchAttribute* at)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nmat * CS);
+    cfg.gridDim = dim3(nmat * cs);
     cfg.blockDim = dim3(JAC_THREADS);
     cfg.dynamicSmemBytes = sm;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CS;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = cs;
+    at->val.clusterDim.y = 1;
+    at->val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (CS > 8) cudaFuncSetAttribute(jacobi_kernel<PER, CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    return cudaLaunchKernelEx(&cfg, jacobi_kernel<PER, CS>, rm, A, V, evals, ldE, work, active, shift, notconv);
+    return cfg;
+}
+
+// Whether the device (a share of one may not) has room for a cluster of
+// 2 JAC_CLUSTER CTAs. It is asked before the launch, not tried by it: a launch
+// that is recorded into a graph succeeds whatever its size, and the graph then
+// fails where nothing can take its place. An error of the two calls is
+// cleared, one that was pending before them is left to the caller.
+template <int PER>
+static bool jacobi_wide_fits(size_t sm)
+{
+    constexpr int cs = 2 * JAC_CLUSTER;
+    const bool clean = cudaPeekAtLastError() == cudaSuccess;
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = jacobi_config(1, cs, sm, nullptr, at);
+    int room = 0;
+    const bool ok =
+        cudaFuncSetAttribute(jacobi_kernel<PER, cs>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+            cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&room, jacobi_kernel<PER, cs>, &cfg) == cudaSuccess;
+    if (!ok && clean) cudaGetLastError();
+    return ok && room > 0;
+}
+
+template <int PER, int CS>
+static void jacobi_cluster(int nmat, cudaStream_t st, size_t sm, const RepMat* rm, const double* A, double* V,
+                           double* evals, int ldE, double* work, const int* active, int shift, int* notconv)
+{
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = jacobi_config(nmat, CS, sm, st, at);
+    cudaLaunchKernelEx(&cfg, jacobi_kernel<PER, CS>, rm, A, V, evals, ldE, work, active, shift, notconv);
 }
 
 template <int PER>
 static void jacobi_launch(int nmat, cudaStream_t st, size_t sm, const RepMat* rm, const double* A, double* V,
                           double* evals, int ldE, double* work, const int* active, int shift, int* notconv)
 {
-    // matrices of 128 or more rows: a cluster of CTAs (SMs) each
+    // matrices of more than 64 rows: a cluster of CTAs (SMs) each
     if constexpr (PER >= 4) {
-        if (nmat <= JAC_FEW) {
-            if (jacobi_cluster<PER, 2 * JAC_CLUSTER>(nmat, st, sm, rm, A, V, evals, ldE, work, active, shift,
-                                                     notconv) == cudaSuccess)
-                return;
-            cudaGetLastError();   // a device share without room for such a cluster: the portable size
-        }
-        jacobi_cluster<PER, JAC_CLUSTER>(nmat, st, sm, rm, A, V, evals, ldE, work, active, shift, notconv);
+        if (nmat <= JAC_FEW && jacobi_wide_fits<PER>(sm))
+            jacobi_cluster<PER, 2 * JAC_CLUSTER>(nmat, st, sm, rm, A, V, evals, ldE, work, active, shift, notconv);
+        else
+            jacobi_cluster<PER, JAC_CLUSTER>(nmat, st, sm, rm, A, V, evals, ldE, work, active, shift, notconv);
     } else {
         jacobi_kernel<PER, 1><<<nmat, JAC_THREADS, sm, st>>>(rm, A, V, evals, ldE, work, active, shift, notconv);
     }
