@@ -162,7 +162,10 @@ __device__ __forceinline__ void prim_quartet(const R* bra, const R* ket, PrimQ<R
 // atom where the quartet has such a pair. The product centres of two tight
 // primitives can then be as close as they are (the integral varies over
 // 1/sqrt(rho)), where a difference of coordinates, or of a centre other than the
-// near one, would leave 2^-48 of a bond length or of the molecule's size.
+// near one, would leave 2^-48 of a bond length or of the molecule's size. X - Y
+// of two atoms is the FP64 difference, made a float-float afterwards: of the
+// coordinates as float-floats it would lose 2^-48 of the distance from the
+// origin, 32 times what FP64 does.
 struct DfCentres {
     int bra, ket;     // first of the three fields P - X: PP_PAX or PP_PBX
     dfloat XY[3];
@@ -173,7 +176,7 @@ struct DfCentres {
         ket = (bra == PP_PAX ? a : b) == d && (bra == PP_PAX ? a : b) != c ? PP_PBX : PP_PAX;
         const int x = bra == PP_PAX ? sa : sb, y = ket == PP_PAX ? sc : sd;
 #pragma unroll
-        for (int k = 0; k < 3; k++) XY[k] = ldg(S.xyzd + 3 * x + k) - ldg(S.xyzd + 3 * y + k);
+        for (int k = 0; k < 3; k++) XY[k] = dfloat(__ldg(S.xyz + 3 * x + k) - __ldg(S.xyz + 3 * y + k));
     }
     // X - Y - (Q - Y) of ket primitive j of pair cd
     __device__ __forceinline__ void ket_part(const Pairs& P, int cd, int j, dfloat aq[3]) const

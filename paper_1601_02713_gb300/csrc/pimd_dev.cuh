@@ -46,7 +46,6 @@ struct Shells {           // all replicas concatenated
     const int* bf;        // first basis function within the replica
     const int* atom;      // global atom index
     const int* rep;       // replica index
-    const dfloat* xyzd;   // xyz as float-floats
 };
 
 struct Pairs {

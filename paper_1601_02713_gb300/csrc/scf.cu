@@ -592,10 +592,7 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
         UPLOAD("sh_src", src, d_src);
         gather_xyz(d_xyz, d_src, nsh, d_shxyz, ctx->stream);
     }
-    dfloat* d_shxyzd;
-    ENSURE("sh_xyzd", (size_t)nsh * 3, d_shxyzd);
-    launch_to_dfloat(d_shxyz, d_shxyzd, (long long)nsh * 3, ctx->stream);
-    bt.S = Shells{d_shxyz, d_l, d_bf, d_satom, d_srep, d_shxyzd};
+    bt.S = Shells{d_shxyz, d_l, d_bf, d_satom, d_srep};
 
     // replicas
     int* d_nbf;

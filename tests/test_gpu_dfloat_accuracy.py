@@ -1,0 +1,108 @@
+"""Error of the float-float kernels on the GPU beside FP64's, for a Fock matrix
+and a two-electron gradient at one fixed density.
+
+An element that the molecule does not hold, with an exponent outside the range
+of the float-float kernels, forces FP64. Tolerance: a float-float operation
+leaves a few 2^-48 of its largest term, so the rounding of a sum stays below
+2^-46 of its norm. The Fock matrix is compared with an unscreened FP64 build's:
+the cutoffs may leave what they leave in FP64. The gradient kernels' cutoffs are
+the FP64 kernels', so there the two are compared with each other."""
+import numpy as np
+import pytest
+
+from paper_1601_02713_gb300 import inputs, native
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+ROUNDING = 2.0 ** -46
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return native.Context(0)
+
+
+def _bases(kind):
+    bas = inputs.basis_set(kind)
+    return native.Basis(bas), native.Basis({**bas, 2: [inputs.Shell(0, [1e9], [1.0])]})
+
+
+def _fock(ctx, B, Z, X, D, tau=1e-12):
+    Dt = torch.tensor(D, device="cuda")
+    G = torch.zeros_like(Dt)
+    native.pimd_fock_dev(ctx, B, Z, X, Dt, G, tau)
+    return G.cpu().numpy()
+
+
+def _density(ctx, B, Z, X):
+    """A few damped Roothaan steps from the core Hamiltonian."""
+    out = []
+    for x in X:
+        S, T, V = native.pimd_one_electron(ctx, B, Z, x)[:3]
+        w, U = np.linalg.eigh(S)
+        L = U / np.sqrt(w)
+        F, D = T + V, None
+        for _ in range(5):
+            C = L @ np.linalg.eigh(L.T @ F @ L)[1][:, :int(Z.sum()) // 2]
+            D = 2.0 * C @ C.T if D is None else C @ C.T + 0.5 * D
+            F = T + V + _fock(ctx, B, Z, x[None], D[None])[0]
+        out.append(D)
+    return np.array(out)
+
+
+class _Device:
+    def __init__(self, ptr, n):
+        self.__cuda_array_interface__ = dict(shape=(n,), typestr="<f8", data=(ptr, False), version=3)
+
+
+def _gradient(ctx, B, Z, X, G, parts=4):
+    """Two-electron gradient at the density of the Fock matrix h + G: one SCF
+    iteration of the force-parallel split, whose reduction puts G in the place
+    of the sum; the shares of all processes but the first, which adds the
+    one-electron part (the tiles are dealt out the same way in every call)."""
+    half = torch.tensor(0.5 * G, device="cuda").reshape(-1)
+    out = []
+
+    def reduce(ptr, n):
+        v = torch.as_tensor(_Device(ptr, n), device="cuda")
+        if n == half.numel():
+            v.copy_(half)
+            torch.cuda.synchronize()
+        else:
+            out.append(v.cpu().numpy().copy())
+
+    for rank in range(1, parts):
+        native.pimd_bo_forces(ctx, B, Z, X, native.scf_opts(guess=0, max_iter=1, split_size=parts, split_rank=rank,
+                                                            reduce=reduce), check=False)
+    return np.sum(out, axis=0)
+
+
+def _check(ctx, kind, Z, X):
+    B, W = _bases(kind)
+    D = _density(ctx, W, Z, X)
+    ref = _fock(ctx, W, Z, X, D, 0.0)
+    df, fp64 = [np.linalg.norm(_fock(ctx, b, Z, X, D) - ref) / np.linalg.norm(ref) for b in (B, W)]
+    assert df < fp64 + ROUNDING
+    df, fp64 = [_gradient(ctx, b, Z, X, ref) for b in (B, W)]
+    assert np.linalg.norm(df - fp64) < ROUNDING * np.linalg.norm(fp64)
+
+
+@pytest.mark.parametrize("offset", [0.0, 100.0, 9000.0])
+def test_no_further_from_exact_than_fp64_at_any_offset(ctx, offset):
+    """Every class of the s/p/d basis, with the molecule at the origin and up to
+    the largest coordinates that the float-float kernels take."""
+    Z, X = inputs.beads(*inputs.water_dimer_geometry(5), 1, 77).stacked()
+    X = np.ascontiguousarray(X + offset * np.array([1.0, -0.7, 0.3]))
+    _check(ctx, "split_spd", Z, X)
+
+
+@pytest.mark.parametrize("kind,nwater", [("min_sp", 1), ("min_sp", 3), ("split_spd", 1), ("split_spd", 4)])
+def test_no_further_from_exact_than_fp64(ctx, kind, nwater):
+    """Both bases, from a molecule of which the cutoffs drop nothing to one of
+    which they drop most."""
+    Z, X = inputs.beads(*inputs.water_cluster_geometry(nwater, 2), 1, 31).stacked()
+    _check(ctx, kind, Z, X)
