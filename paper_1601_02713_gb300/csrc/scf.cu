@@ -981,6 +981,14 @@ static std::vector<std::pair<int, int>> class_jobs(const Batch& bt, IsDf&& is_df
 // asks for a primitive cutoff below kDfMinPrim (the default is 1e-12 / 81 =
 // 1.23e-14) wants a smaller error than that rounding: everything in FP64 then.
 constexpr double kDfTau = 1e-2, kDfMinPrim = 1.2e-14;
+// The same for the gradient, whose bound Q_ab Q_cd |Gamma| carries no derivative
+// scale: the derivative integrals are up to some 1e2 times larger (2 sqrt(2
+// exponent)). Float-float minus FP64 gradient at one density and the same cutoffs
+// with a bound of 1e-2 / 1e-3 / 1e-4, beside the distance of two FP64 calls
+// (hartree per bohr, norms): 2 H2O 5.7e-14 / 1.7e-14 / 1.6e-14, 4.3e-14; (H2O)8
+// 9.3e-13 / 1.5e-13 / 1.4e-13, 8.7e-13; a Diels-Alder image 1.1e-12 / 7.3e-13 /
+// 3.9e-13, 2.2e-12. The gradient of 4 (H2O)8 beads takes 869 / 870 / 877 ms.
+constexpr double kDfTauGrad = 1e-4;
 // The bound below which a build with these cutoffs runs in float-floats, 0: none
 static double df_bound(const Batch& bt, double df_tau, double tau, double fp32_tau, double tau_prim)
 {
@@ -1559,7 +1567,7 @@ static int run_batch(pimd_ctx* ctx, int nrep, const int* natom_of, const int* Zc
         }
         CK(cudaEventRecord(ctx->ev[4], ctx->stream));
         launch_shell_bounds(bt.S, bt.R, nrep, bt.maxsh, m.D, bt.Dsh, nullptr, ctx->stream);
-        DfBuild df{df_bound(bt, kDfTau, o->schwarz_tau * 1e-2, o->fp32_tau, o->schwarz_tau * o->prim_screen), 0, Md,
+        DfBuild df{df_bound(bt, kDfTauGrad, o->schwarz_tau * 1e-2, o->fp32_tau, o->schwarz_tau * o->prim_screen), 0, Md,
                    ctx->boysd};
         if (df.tau > 0.0) {
             launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);
@@ -1943,7 +1951,7 @@ extern "C" int pimd_autotune(pimd_ctx* ctx, int nrep, int natom, const int* Z, c
         if (!rc2) rc2 = dev_ensure(ctx, "tune_grad", (size_t)nrep * natom * 3, &d_g);
         if (!rc2) {
             launch_shell_bounds(bt.S, bt.R, nrep, bt.maxsh, m.D, bt.Dsh, nullptr, ctx->stream);
-            DfBuild df{df_bound(bt, kDfTau, o.schwarz_tau * 1e-2, o.fp32_tau, o.schwarz_tau * o.prim_screen), 0,
+            DfBuild df{df_bound(bt, kDfTauGrad, o.schwarz_tau * 1e-2, o.fp32_tau, o.schwarz_tau * o.prim_screen), 0,
                        nullptr, ctx->boysd};
             dfloat* Md = nullptr;
             rc2 = dev_ensure(ctx, "Md", (size_t)bt.mtot, &Md);

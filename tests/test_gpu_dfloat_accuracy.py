@@ -59,11 +59,12 @@ class _Device:
         self.__cuda_array_interface__ = dict(shape=(n,), typestr="<f8", data=(ptr, False), version=3)
 
 
-def _gradient(ctx, B, Z, X, G, parts=4):
+def _gradient(ctx, B, Z, X, G, parts=4, first=1):
     """Two-electron gradient at the density of the Fock matrix h + G: one SCF
     iteration of the force-parallel split, whose reduction puts G in the place
     of the sum; the shares of all processes but the first, which adds the
-    one-electron part (the tiles are dealt out the same way in every call)."""
+    one-electron part (first = 0: with it). The tiles are dealt out the same way
+    in every call."""
     half = torch.tensor(0.5 * G, device="cuda").reshape(-1)
     out = []
 
@@ -75,7 +76,7 @@ def _gradient(ctx, B, Z, X, G, parts=4):
         else:
             out.append(v.cpu().numpy().copy())
 
-    for rank in range(1, parts):
+    for rank in range(first, parts):
         native.pimd_bo_forces(ctx, B, Z, X, native.scf_opts(guess=0, max_iter=1, split_size=parts, split_rank=rank,
                                                             reduce=reduce), check=False)
     return np.sum(out, axis=0)
@@ -106,3 +107,16 @@ def test_no_further_from_exact_than_fp64(ctx, kind, nwater):
     which they drop most."""
     Z, X = inputs.beads(*inputs.water_cluster_geometry(nwater, 2), 1, 31).stacked()
     _check(ctx, kind, Z, X)
+
+
+def test_gradient_rounding_below_that_of_fp64(ctx):
+    """The float-float part adds less than half of the distance between two FP64
+    gradients (FP64 atomics in another order) at one density: an independent
+    error of that size raises the whole by an eighth."""
+    Z, X = inputs.beads(*inputs.water_cluster_geometry(8, 2), 1, 2064).stacked()
+    B, W = _bases("split_spd")
+    ref = _fock(ctx, W, Z, X, _density(ctx, W, Z, X))
+    whole = [_gradient(ctx, W, Z, X, ref, first=0) for _ in range(3)]
+    spread = np.mean([np.linalg.norm(whole[i] - whole[i - 1]) for i in range(3)])
+    df, fp64 = [np.mean([_gradient(ctx, b, Z, X, ref) for _ in range(3)], axis=0) for b in (B, W)]
+    assert np.linalg.norm(df - fp64) < 0.5 * spread
