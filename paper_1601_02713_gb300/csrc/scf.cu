@@ -978,9 +978,10 @@ static std::vector<std::pair<int, int>> class_jobs(const Batch& bt, IsDf&& is_df
 // 2.58e-13, (H2O)16 1.02e-12 -> 1.02e-12, one H2O 9.55e-15 -> 9.43e-15 (without
 // any cutoff 4e-16 / 4e-16 / 1e-15 / 9e-17 -> 1.6e-14 / 2.1e-14 / 1.2e-14 /
 // 1.2e-15; DF_TAU_PRIM makes up for that at the default cutoffs). A caller who
-// asks for a primitive cutoff below kDfMinPrim (the default is 1e-12 / 81 =
-// 1.23e-14) wants a smaller error than that rounding: everything in FP64 then.
-constexpr double kDfTau = 1e-2, kDfMinPrim = 1.2e-14;
+// asks for a quartet cutoff below the default kDfMinTau or a primitive cutoff
+// below kDfMinPrim (the default is 1e-12 / 81 = 1.23e-14) wants a smaller error
+// than that rounding: everything in FP64 then.
+constexpr double kDfTau = 1e-2, kDfMinTau = 1e-12, kDfMinPrim = 1.2e-14;
 // The same for the gradient, whose bound Q_ab Q_cd |Gamma| carries no derivative
 // scale: the derivative integrals are up to some 1e2 times larger (2 sqrt(2
 // exponent)). Float-float minus FP64 gradient at one density and the same cutoffs
@@ -990,9 +991,13 @@ constexpr double kDfTau = 1e-2, kDfMinPrim = 1.2e-14;
 // 3.9e-13, 2.2e-12. The gradient of 4 (H2O)8 beads takes 869 / 870 / 877 ms.
 constexpr double kDfTauGrad = 1e-4;
 // The bound below which a build with these cutoffs runs in float-floats, 0: none
-static double df_bound(const Batch& bt, double df_tau, double tau, double fp32_tau, double tau_prim)
+// (schwarz_tau, tau_prim: the caller's; tau: the kernels' quartet cutoff, in the
+// gradient a hundredth of schwarz_tau)
+static double df_bound(const Batch& bt, double df_tau, double schwarz_tau, double tau_prim, double tau,
+                       double fp32_tau)
 {
-    return bt.df_ok && tau_prim >= kDfMinPrim && df_tau > std::max(tau, fp32_tau) ? df_tau : 0.0;
+    return bt.df_ok && schwarz_tau >= kDfMinTau && tau_prim >= kDfMinPrim && df_tau > std::max(tau, fp32_tau) ? df_tau
+                                                                                                              : 0.0;
 }
 
 // G' += G'(M) over all class pairs for the replicas in the active mask, with
@@ -1011,7 +1016,7 @@ static int fock_build(pimd_ctx* ctx, Batch& bt, Mats& m, double tau, double fp32
         launch_to_float(M, Mf, bt.mtot, ctx->stream);
         ctx->stats.kernel_launches++;
     }
-    DfBuild df{df_bound(bt, df_tau, tau, fp32_tau, tau_prim), 0, nullptr, ctx->boysd};
+    DfBuild df{df_bound(bt, df_tau, tau, tau_prim, tau, fp32_tau), 0, nullptr, ctx->boysd};
     if (df.tau > 0.0) {
         dfloat* Md;
         ENSURE("Md", bt.mtot, Md);
@@ -1567,8 +1572,9 @@ static int run_batch(pimd_ctx* ctx, int nrep, const int* natom_of, const int* Zc
         }
         CK(cudaEventRecord(ctx->ev[4], ctx->stream));
         launch_shell_bounds(bt.S, bt.R, nrep, bt.maxsh, m.D, bt.Dsh, nullptr, ctx->stream);
-        DfBuild df{df_bound(bt, kDfTauGrad, o->schwarz_tau * 1e-2, o->fp32_tau, o->schwarz_tau * o->prim_screen), 0, Md,
-                   ctx->boysd};
+        DfBuild df{df_bound(bt, kDfTauGrad, o->schwarz_tau, o->schwarz_tau * o->prim_screen, o->schwarz_tau * 1e-2,
+                            o->fp32_tau),
+                   0, Md, ctx->boysd};
         if (df.tau > 0.0) {
             launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);
             ctx->stats.kernel_launches++;
@@ -1918,8 +1924,8 @@ extern "C" int pimd_autotune(pimd_ctx* ctx, int nrep, int natom, const int* Z, c
         cudaMemsetAsync(m.G, 0, sizeof(double) * bt.mtot, ctx->stream);
         launch_shell_bounds(bt.S, bt.R, bt.nrep, bt.maxsh, m.D, bt.Dsh, bt.R.active, ctx->stream);
         if (Mf) launch_to_float(m.D, Mf, bt.mtot, ctx->stream);
-        DfBuild df{df_bound(bt, kDfTau, o.schwarz_tau, o.fp32_tau, o.schwarz_tau * o.prim_screen), 0, nullptr,
-                   ctx->boysd};
+        DfBuild df{df_bound(bt, kDfTau, o.schwarz_tau, o.schwarz_tau * o.prim_screen, o.schwarz_tau, o.fp32_tau), 0,
+                   nullptr, ctx->boysd};
         dfloat* Md;
         if ((rc2 = dev_ensure(ctx, "Md", (size_t)bt.mtot, &Md))) break;
         launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);
@@ -1951,8 +1957,9 @@ extern "C" int pimd_autotune(pimd_ctx* ctx, int nrep, int natom, const int* Z, c
         if (!rc2) rc2 = dev_ensure(ctx, "tune_grad", (size_t)nrep * natom * 3, &d_g);
         if (!rc2) {
             launch_shell_bounds(bt.S, bt.R, nrep, bt.maxsh, m.D, bt.Dsh, nullptr, ctx->stream);
-            DfBuild df{df_bound(bt, kDfTauGrad, o.schwarz_tau * 1e-2, o.fp32_tau, o.schwarz_tau * o.prim_screen), 0,
-                       nullptr, ctx->boysd};
+            DfBuild df{df_bound(bt, kDfTauGrad, o.schwarz_tau, o.schwarz_tau * o.prim_screen, o.schwarz_tau * 1e-2,
+                                o.fp32_tau),
+                       0, nullptr, ctx->boysd};
             dfloat* Md = nullptr;
             rc2 = dev_ensure(ctx, "Md", (size_t)bt.mtot, &Md);
             if (!rc2) launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);

@@ -120,3 +120,18 @@ def test_gradient_rounding_below_that_of_fp64(ctx):
     spread = np.mean([np.linalg.norm(whole[i] - whole[i - 1]) for i in range(3)])
     df, fp64 = [np.mean([_gradient(ctx, b, Z, X, ref) for _ in range(3)], axis=0) for b in (B, W)]
     assert np.linalg.norm(df - fp64) < 0.5 * spread
+
+
+@pytest.mark.parametrize("tau,prim,fp64", [(1e-13, 0.2, True), (0.99e-12, 1.0, True), (1e-12, 1.0, False),
+                                           (1e-12, 1.0 / 81.0, False), (1e-12, 0.01, True)])
+def test_a_tighter_cutoff_of_either_kind_keeps_fp64(ctx, tau, prim, fp64):
+    """Launch for launch the calls of the basis that is outside the range."""
+    Z, X = inputs.beads(*inputs.water_cluster_geometry(1, 2), 1, 5).stacked()
+
+    def launches(b):
+        native.pimd_bo_forces(ctx, b, Z, X, native.scf_opts(guess=0, max_iter=2, schwarz_tau=tau, prim_screen=prim),
+                              check=False)
+        return native.pimd_last_stats(ctx)["kernel_launches"]   # of the last forces call
+
+    B, W = _bases("split_spd")
+    assert (launches(B) == launches(W)) == fp64
