@@ -138,16 +138,16 @@ def generate_sources():
             e += _coop_upload_code(nm, False, g)
         # bs > 0: straight-line kernel with bs threads per block; bs == 0: the
         # cooperative tape kernel
-        e += [f"void launch_jk_{nm}(const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles,",
+        e += [f"int launch_jk_{nm}(const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles,",
               "                     const double* D, const float* Df, const DfBuild& df, double* G, const double* boys,",
               "                     const float* boysf, double tau, double fp32_tau, const double* Dsh,",
               "                     unsigned long long* cnt, int bs, double tp, double fxs, cudaStream_t st)",
               "{",
-              "    if (ntiles <= 0) return;",
+              "    if (ntiles <= 0) return 0;",
               "    const double split = fp32_tau > tau ? fp32_tau : tau;"]
         if coop_e[nm]:
             e += [f"    if (bs == 0{'' if straight_e[nm] else ' || true'}) {{",
-                  "        if (df.stage == 1) return;",
+                  "        if (df.stage == 1) return 0;",
                   "        CoopTape t; int W, Wf; size_t bytes, bytesf;",
                   f"        coop_tape_{nm}(t, W, bytes, Wf, bytesf);",
                   "        const dim3 grid(ntiles, coop_blocks_per_tile(ntiles));",
@@ -156,25 +156,33 @@ def generate_sources():
                   "        if (fp32_tau > tau)",
                   f"            jk_coop_kernel<{la}, {lb}, {lc}, {ld}, float><<<grid, 32 * Wf, bytesf, st>>>(P, S, R,",
                   "                tiles, Df, G, boysf, tau, fp32_tau, Dsh, cnt + 2, t, tp, fxs);",
-                  "        return;",
+                  "        return fp32_tau > tau ? 2 : 1;",
                   "    }"]
         if straight_e[nm]:
             e += ["    const int b = bs > 0 ? bs : 128;",
                   "    const dim3 grid(ntiles, jk_blocks_per_tile(ntiles));"]
             top = "1e300" if df_all[nm] else "df.tau"
             e += [f"    const double top = df.tau > split ? {top} : split;",
-                  "    if (top > split && df.stage != 2)",
+                  "    int n = 0;",
+                  "    if (top > split && df.stage != 2) {",
                   f"        jk_kernel<Cls_{nm}, dfloat><<<grid, b, 0, st>>>(P, S, R, tiles,",
                   f"                                                        tail_density<Cls_{nm}>(D, df.D), G,",
                   "                                                        df.boys, split, top, Dsh, cnt, DF_TAU_PRIM * tp,",
                   "                                                        fxs);",
-                  "    if (df.stage == 1) return;",
-                  "    if (top < 1e300)",
+                  "        n++;",
+                  "    }",
+                  "    if (df.stage == 1) return n;",
+                  "    if (top < 1e300) {",
                   f"        jk_kernel<Cls_{nm}, double><<<grid, b, 0, st>>>(P, S, R, tiles, D, G, boys, top, 1e300, Dsh, cnt,",
                   "                                                      tp, fxs);",
-                  "    if (fp32_tau > tau)",
+                  "        n++;",
+                  "    }",
+                  "    if (fp32_tau > tau) {",
                   f"        jk_kernel<Cls_{nm}, float><<<ntiles, b, 0, st>>>(P, S, R, tiles, Df, G, boysf, tau, fp32_tau, Dsh,",
-                  "                                                       cnt + 2, tp, fxs);"]
+                  "                                                       cnt + 2, tp, fxs);",
+                  "        n++;",
+                  "    }",
+                  "    return n;"]
         e.append("}")
         if same:
             e += [f"void launch_schwarz_{nm}(const Pairs& P, const Shells& S, const int* list, int n,",
@@ -201,17 +209,17 @@ def generate_sources():
         else:
             gl.append(f"void grad2e_upload_{nm}() {{}}")
         # variant 0: cooperative tape kernel, 1: straight-line kernel with bs threads
-        gl += [f"void launch_grad2e_{nm}(const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles,",
+        gl += [f"int launch_grad2e_{nm}(const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles,",
                "                        const double* D, const DfBuild& df, double* grad, const double* boys,",
                "                        const float* boysf,",
                "                        double tau, double fp32_tau, const double* Dsh, unsigned long long* cnt,",
                "                        int variant, int bs, double tp, double fxs, cudaStream_t st)",
                "{",
-               "    if (ntiles <= 0) return;",
+               "    if (ntiles <= 0) return 0;",
                "    const double split = fp32_tau > tau ? fp32_tau : tau;"]
         if coop_g[nm]:
             gl += [f"    if (variant == 0{' || true' if heavy[nm] else ''}) {{",
-                   "        if (df.stage == 1) return;",
+                   "        if (df.stage == 1) return 0;",
                    "        CoopTape t; int W, Wf; size_t bytes, bytesf;",
                    f"        coop_tape_{nm}(t, W, bytes, Wf, bytesf);",
                    "        const dim3 grid(ntiles, coop_blocks_per_tile(ntiles));",
@@ -220,24 +228,31 @@ def generate_sources():
                    "        if (fp32_tau > tau)",
                    f"            grad2e_coop_kernel<{la}, {lb}, {lc}, {ld}, float><<<grid, 32 * Wf, bytesf, st>>>(P, S,",
                    "                R, tiles, D, grad, boysf, tau, fp32_tau, Dsh, cnt + 2, t, tp, fxs);",
-                   "        return;",
+                   "        return fp32_tau > tau ? 2 : 1;",
                    "    }"]
         if not heavy[nm]:
             gl += ["    const int b = bs > 0 ? bs : 128;",
-                   "    const dim3 grid(ntiles, jk_blocks_per_tile(ntiles));"]
+                   "    const dim3 grid(ntiles, jk_blocks_per_tile(ntiles));",
+                   "    int n = 0;"]
             if df_g[nm]:
                 gl += ["    const double top = df.tau > split ? df.tau : split;",
-                       "    if (top > split && df.stage != 2)",
+                       "    if (top > split && df.stage != 2) {",
                        f"        grad2e_kernel<GCls_{nm}, dfloat><<<grid, b, 0, st>>>(P, S, R, tiles, df.D, grad, df.boys,",
-                       "                                                            split, top, Dsh, cnt, tp, fxs);"]
+                       "                                                            split, top, Dsh, cnt, tp, fxs);",
+                       "        n++;",
+                       "    }"]
             else:
                 gl += ["    const double top = split;"]
-            gl += ["    if (df.stage == 1) return;",
+            gl += ["    if (df.stage == 1) return n;",
                    f"    grad2e_kernel<GCls_{nm}, double><<<grid, b, 0, st>>>(P, S, R, tiles, D, grad, boys, top, 1e300, Dsh,",
                    "                                                            cnt, tp, fxs);",
-                   "    if (fp32_tau > tau)",
+                   "    n++;",
+                   "    if (fp32_tau > tau) {",
                    f"        grad2e_kernel<GCls_{nm}, float><<<ntiles, b, 0, st>>>(P, S, R, tiles, D, grad, boysf, tau, fp32_tau,",
-                   "                                                           Dsh, cnt + 2, tp, fxs);"]
+                   "                                                           Dsh, cnt + 2, tp, fxs);",
+                   "        n++;",
+                   "    }",
+                   "    return n;"]
         gl.append("}")
         gl.append("}  // namespace pimd\n")
         p = os.path.join(GEN, f"tu_grad_{nm}.cu")
@@ -253,11 +268,11 @@ def generate_sources():
     sig_g = ("const Pairs&, const Shells&, const Reps&, const Tile*, int, const double*, const DfBuild&, double*, "
              "const double*, const float*, double, double, const double*, unsigned long long*, int, int, double, double, cudaStream_t")
     for c, nm in zip(classes, names):
-        d.append(f"void launch_jk_{nm}({sig_jk});")
+        d.append(f"int launch_jk_{nm}({sig_jk});")
         if (c[0], c[1]) == (c[2], c[3]):
             d.append(f"void launch_schwarz_{nm}({sig_sw});")
             d.append(f"void launch_prim_schwarz_{nm}({sig_psw});")
-        d.append(f"void launch_grad2e_{nm}({sig_g});")
+        d.append(f"int launch_grad2e_{nm}({sig_g});")
         d.append(f"void grad2e_upload_{nm}();")
     d.append(f"int n_class_pairs() {{ return {len(classes)}; }}")
     d.append("void class_pair_ls(int cp, int* la, int* lb, int* lc, int* ld)")
@@ -286,13 +301,13 @@ def generate_sources():
                                                         for c, nm in zip(classes, names)) + "};")
     d.append("    return t[cp];")
     d.append("}")
-    d.append(f"typedef void (*JkFn)({sig_jk});")
+    d.append(f"typedef int (*JkFn)({sig_jk});")
     d.append("static const JkFn jk_tab[] = {" + ", ".join(f"launch_jk_{nm}" for nm in names) + "};")
-    d.append("void launch_jk(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles, "
+    d.append("int launch_jk(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles, "
              "const double* D, const float* Df, const DfBuild& df, double* G, const double* boys, const float* boysf, "
              "double tau, double fp32_tau, const double* Dsh, unsigned long long* cnt, int bs, double tau_prim, "
              "double fxs, cudaStream_t st)")
-    d.append("{ jk_tab[cp](P, S, R, tiles, ntiles, D, Df, df, G, boys, boysf, tau, fp32_tau, Dsh, cnt, bs, tau_prim, fxs, st); }")
+    d.append("{ return jk_tab[cp](P, S, R, tiles, ntiles, D, Df, df, G, boys, boysf, tau, fp32_tau, Dsh, cnt, bs, tau_prim, fxs, st); }")
     for fn, tab in (("class_pair_coop", coop_e), ("class_pair_straight", straight_e), ("grad_pair_coop", coop_g),
                     ("class_pair_df", df_e), ("class_pair_df_all", df_all), ("grad_pair_df", df_g),
                     ("grad_pair_straight", {nm: not heavy[nm] for nm in names})):
@@ -312,14 +327,14 @@ def generate_sources():
     d.append("void launch_prim_schwarz(int X, const Pairs& P, const Shells& S, const int* list, int n, "
              "const double* boys, double* pp, float* qp, float* qg, cudaStream_t st)")
     d.append("{ psw_tab[X](P, S, list, n, boys, pp, qp, qg, st); }")
-    d.append(f"typedef void (*GFn)({sig_g});")
+    d.append(f"typedef int (*GFn)({sig_g});")
     d.append("static const GFn g_tab[] = {" + ", ".join(f"launch_grad2e_{nm}" for nm in names) + "};")
 
-    d.append("void launch_grad2e(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles, "
+    d.append("int launch_grad2e(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles, "
              "const double* D, const DfBuild& df, double* grad, const double* boys, const float* boysf, double tau, "
              "double fp32_tau, const double* Dsh, unsigned long long* cnt, int variant, int bs, double tau_prim, double fxs, "
              "cudaStream_t st)")
-    d.append("{ g_tab[cp](P, S, R, tiles, ntiles, D, df, grad, boys, boysf, tau, fp32_tau, Dsh, cnt, variant, bs, tau_prim, "
+    d.append("{ return g_tab[cp](P, S, R, tiles, ntiles, D, df, grad, boys, boysf, tau, fp32_tau, Dsh, cnt, variant, bs, tau_prim, "
              "fxs, st); }")
     d.append("void grad2e_tapes_upload() {")
     for nm in names:

@@ -65,6 +65,7 @@ long long class_grad_flops(int cp);   // per primitive quartet of the gradient
 // ignores the choice)
 // tau_prim: primitive quartets with qp_i qp_j max|D block| below it are skipped (0: none)
 // fxs > 0: G accumulated as fixed-point integers scaled by fxs (deterministic mode, det_add)
+// returns the number of kernels launched (launch_grad2e as well)
 // df: of the FP64 part, quartets with bound < df.tau run in float-float
 // arithmetic (dfloat.cuh) where the class has a straight-line kernel
 struct DfBuild {
@@ -73,10 +74,10 @@ struct DfBuild {
     const dfloat* D;      // the density as float-floats
     const dfloat* boys;   // the FP64 Boys table as float-floats
 };
-void launch_jk(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles,
-               const double* D, const float* Df, const DfBuild& df, double* G, const double* boys,
-               const float* boysf, double tau, double fp32_tau, const double* Dsh, unsigned long long* cnt, int bs,
-               double tau_prim, double fxs, cudaStream_t st);
+int launch_jk(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles,
+              const double* D, const float* Df, const DfBuild& df, double* G, const double* boys,
+              const float* boysf, double tau, double fp32_tau, const double* Dsh, unsigned long long* cnt, int bs,
+              double tau_prim, double fxs, cudaStream_t st);
 // kernel variants generated for a class pair: the cooperative tape
 // kernel and the straight-line kernel, for the Fock build and the gradient
 bool class_pair_coop(int cp);
@@ -98,7 +99,7 @@ void launch_prim_schwarz(int pair_class, const Pairs& P, const Shells& S, const 
 // block (a class with one variant ignores the choice)
 // (tau_prim: primitive quartets with (qg_i qp_j + qp_i qg_j) |Gamma| below it are skipped; 0 none)
 // cnt[0..1]: executed FP64 quartets and primitive quartets, cnt[2..3] FP32
-void launch_grad2e(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles,
+int launch_grad2e(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile* tiles, int ntiles,
                    const double* D, const DfBuild& df, double* grad, const double* boys, const float* boysf, double tau,
                    double fp32_tau, const double* Dsh, unsigned long long* cnt, int variant, int bs,
                    double tau_prim, double fxs, cudaStream_t st);

@@ -1031,9 +1031,9 @@ static int fock_build(pimd_ctx* ctx, Batch& bt, Mats& m, double tau, double fp32
         const int cp = jobs[k].first;
         DfBuild d = df;
         d.stage = jobs[k].second;
-        launch_jk(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), M, Mf, d, m.G, ctx->boys,
-                  ctx->boysf, tau, fp32_tau, bt.Dsh, bt.cnt + 4 * cp, ctx->tile_w[cp], tau_prim, fxs, st);
-        ctx->stats.kernel_launches += 1 + (fp32_tau > tau && d.stage != 1);
+        ctx->stats.kernel_launches +=
+            launch_jk(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), M, Mf, d, m.G, ctx->boys,
+                      ctx->boysf, tau, fp32_tau, bt.Dsh, bt.cnt + 4 * cp, ctx->tile_w[cp], tau_prim, fxs, st);
     });
     if (rc) return rc;
     if (fxs > 0) {
@@ -1584,12 +1584,12 @@ static int run_batch(pimd_ctx* ctx, int nrep, const int* natom_of, const int* Zc
             const int cp = jobs[k].first;
             DfBuild d = df;
             d.stage = jobs[k].second;
-            launch_grad2e(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), m.D, d, d_grad, ctx->boys,
-                          ctx->boysf, o->schwarz_tau * 1e-2, o->fp32_tau, bt.Dsh, bt.cnt + 4 * 64 + 4 * cp,
-                          ctx->grad_var[cp],
-                          ctx->tile_w[cp] > 0 ? ctx->tile_w[cp] : 128, o->schwarz_tau * o->prim_screen,
-                          fx_grad, st);
-            ctx->stats.kernel_launches += 1 + (o->fp32_tau > 0 && d.stage != 1);
+            ctx->stats.kernel_launches +=
+                launch_grad2e(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), m.D, d, d_grad,
+                              ctx->boys, ctx->boysf, o->schwarz_tau * 1e-2, o->fp32_tau, bt.Dsh,
+                              bt.cnt + 4 * 64 + 4 * cp, ctx->grad_var[cp],
+                              ctx->tile_w[cp] > 0 ? ctx->tile_w[cp] : 128, o->schwarz_tau * o->prim_screen, fx_grad,
+                              st);
         });
         if (rcg) return rcg;
         CK(cudaEventRecord(ctx->ev[5], ctx->stream));

@@ -135,3 +135,36 @@ def test_a_tighter_cutoff_of_either_kind_keeps_fp64(ctx, tau, prim, fp64):
 
     B, W = _bases("split_spd")
     assert (launches(B) == launches(W)) == fp64
+
+
+def _profiled(fn):
+    """(fn(), kernels that ran on the device meanwhile)"""
+    from torch.profiler import ProfilerActivity, profile
+
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as p:
+        out = fn()
+        torch.cuda.synchronize()
+    return out, sum(1 for e in p.events() if "_kernel" in e.name)
+
+
+@pytest.mark.parametrize("fp32_tau", [0.0, 1e-15, 1e-6])
+def test_launch_counter_counts_what_runs(ctx, fp32_tau):
+    """The counter's difference between the float-float and the FP64 form of a
+    call is that of the kernels seen by the profiler, in FP64 and mixed
+    precision, and for an FP32 bound below the gradient's quartet cutoff (no
+    FP32 launch)."""
+    Z, X = inputs.beads(*inputs.water_cluster_geometry(1, 2), 1, 5).stacked()
+
+    def launches(b, f):
+        native.pimd_bo_forces(ctx, b, Z, X, native.scf_opts(guess=0, max_iter=1, use_graphs=0, fp32_tau=f),
+                              check=False)
+        return native.pimd_last_stats(ctx)["kernel_launches"]
+
+    B, W = _bases("split_spd")
+    launches(B, fp32_tau)
+    _profiled(lambda: launches(W, 0.0))   # one-time set-up of the library and of the profiler
+    n0, seen0 = _profiled(lambda: launches(W, 0.0))
+    n1, seen1 = _profiled(lambda: launches(B, fp32_tau))
+    assert seen0 > 40
+    assert n1 - n0 == seen1 - seen0
