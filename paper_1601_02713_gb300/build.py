@@ -121,7 +121,6 @@ def generate_sources():
     coop_e = {s[0]: s[7] for s in stats}
     coop_g = {s[0]: s[8] for s in stats}
     straight_e = {s[0]: s[9] for s in stats}
-    df_e = straight_e   # every straight-line class has a float-float Fock kernel
     df_g = {s[0]: s[10] for s in stats}
     df_all = {s[0]: s[11] for s in stats}
     classes = g.classes()
@@ -161,7 +160,7 @@ def generate_sources():
         if straight_e[nm]:
             e += ["    const int b = bs > 0 ? bs : 128;",
                   "    const dim3 grid(ntiles, jk_blocks_per_tile(ntiles));"]
-            top = "1e300" if df_all[nm] else "df.tau"
+            top = "df.tau_all" if df_all[nm] else "df.tau"
             e += [f"    const double top = df.tau > split ? {top} : split;",
                   "    int n = 0;",
                   "    if (top > split && df.stage != 2) {",
@@ -172,11 +171,9 @@ def generate_sources():
                   "        n++;",
                   "    }",
                   "    if (df.stage == 1) return n;",
-                  "    if (top < 1e300) {",
-                  f"        jk_kernel<Cls_{nm}, double><<<grid, b, 0, st>>>(P, S, R, tiles, D, G, boys, top, 1e300, Dsh, cnt,",
-                  "                                                      tp, fxs);",
-                  "        n++;",
-                  "    }",
+                  f"    jk_kernel<Cls_{nm}, double><<<grid, b, 0, st>>>(P, S, R, tiles, D, G, boys, top, 1e300, Dsh, cnt,",
+                  "                                                    tp, fxs);",
+                  "    n++;",
                   "    if (fp32_tau > tau) {",
                   f"        jk_kernel<Cls_{nm}, float><<<ntiles, b, 0, st>>>(P, S, R, tiles, Df, G, boysf, tau, fp32_tau, Dsh,",
                   "                                                       cnt + 2, tp, fxs);",
@@ -309,7 +306,7 @@ def generate_sources():
              "double fxs, cudaStream_t st)")
     d.append("{ return jk_tab[cp](P, S, R, tiles, ntiles, D, Df, df, G, boys, boysf, tau, fp32_tau, Dsh, cnt, bs, tau_prim, fxs, st); }")
     for fn, tab in (("class_pair_coop", coop_e), ("class_pair_straight", straight_e), ("grad_pair_coop", coop_g),
-                    ("class_pair_df", df_e), ("class_pair_df_all", df_all), ("grad_pair_df", df_g),
+                    ("grad_pair_df", df_g),
                     ("grad_pair_straight", {nm: not heavy[nm] for nm in names})):
         d.append(f"bool {fn}(int cp)")
         d.append("{")

@@ -675,10 +675,11 @@ def encode_hrr(op):
 COOP_ENERGY_MIN_VRR = 2000
 STRAIGHT_ENERGY_MAX_VRR = 2000
 COOP_GRAD_MIN_VRR = 400
-# Fock classes above this many operations per primitive quartet run all their
-# FP64 quartets in float-float arithmetic: a launch for their few largest ones
-# cost as much as a tenth of the class (FP64 (dd|dp) quartets above 1e-2 of 4
-# (H2O)8 beads: 18 ms beside 16 ms for the rest in float-float).
+# Fock classes above this many operations per primitive quartet run (nearly) all
+# their FP64 quartets in float-float arithmetic, up to the bound tau_all: a launch
+# for the few largest ones cost as much as a tenth of the class (FP64 (dd|dp)
+# quartets above 1e-2 of 4 (H2O)8 beads: 18 ms beside 16 ms for the rest in
+# float-float).
 DF_ALL_MIN_FLOPS = 1000
 # float-float gradient kernel: up to this many operations per primitive quartet.
 # The gradient's recursion runs to order L + 1 into four accumulator sets, and

@@ -70,6 +70,7 @@ long long class_grad_flops(int cp);   // per primitive quartet of the gradient
 // arithmetic (dfloat.cuh) where the class has a straight-line kernel
 struct DfBuild {
     double tau;           // 0: none
+    double tau_all;       // the same for the Fock classes with long recursions
     int stage;            // 0: all launches; 1: the float-float ones; 2: the others
     const dfloat* D;      // the density as float-floats
     const dfloat* boys;   // the FP64 Boys table as float-floats
@@ -82,8 +83,6 @@ int launch_jk(int cp, const Pairs& P, const Shells& S, const Reps& R, const Tile
 // kernel and the straight-line kernel, for the Fock build and the gradient
 bool class_pair_coop(int cp);
 bool class_pair_straight(int cp);
-bool class_pair_df(int cp);
-bool class_pair_df_all(int cp);   // every FP64 quartet of the class runs in float-float arithmetic
 bool grad_pair_df(int cp);
 bool grad_pair_coop(int cp);
 bool grad_pair_straight(int cp);

@@ -969,19 +969,24 @@ static std::vector<std::pair<int, int>> class_jobs(const Batch& bt, IsDf&& is_df
 
 // The FP64 quartets whose density-weighted bound is below this run in
 // float-float arithmetic (dfloat.cuh; not for shell exponents or coordinates
-// outside its range), in the classes with long recursions all of them
-// (class_pair_df_all; their integrals are not the largest). The rounding error
-// of a few 1e-14 of an integral is then of the order of what FP64 leaves in the
-// largest integrals, and below the integral cutoffs' error. Error of the Fock
-// matrix against an unscreened FP64 build in units of its norm, all in FP64 ->
-// with this: 4 (H2O)8 beads 5.31e-13 -> 5.28e-13, a Diels-Alder image 2.67e-13 ->
-// 2.58e-13, (H2O)16 1.02e-12 -> 1.02e-12, one H2O 9.55e-15 -> 9.43e-15 (without
-// any cutoff 4e-16 / 4e-16 / 1e-15 / 9e-17 -> 1.6e-14 / 2.1e-14 / 1.2e-14 /
-// 1.2e-15; DF_TAU_PRIM makes up for that at the default cutoffs). A caller who
-// asks for a quartet cutoff below the default kDfMinTau or a primitive cutoff
-// below kDfMinPrim (the default is 1e-12 / 81 = 1.23e-14) wants a smaller error
-// than that rounding: everything in FP64 then.
-constexpr double kDfTau = 1e-2, kDfMinTau = 1e-12, kDfMinPrim = 1.2e-14;
+// outside its range). Their rounding is then of the order of what FP64 leaves in
+// the largest integrals, and below the integral cutoffs' error. In the classes
+// with long recursions, whose rounding is 2^-46 to 2^-43 of a quartet, the bound
+// is kDfAll times the quartet cutoff: what a quartet's rounding leaves stays below
+// the cutoff, that is below what a skipped quartet may leave. Densities of
+// molecules stay far below it; a density scaled up to where the cutoffs no longer
+// matter goes to FP64 (two p/d atoms with nothing screened, a dense density of
+// order 10: without the bound 1e-13 of the norm, FP64 3e-16).
+// Error of the Fock matrix against an unscreened FP64 build in units of its norm,
+// all in FP64 -> with this: 1 to 16 H2O in the s/p/d basis 2.2e-14 -> 1.7e-14,
+// 9.0e-14 -> 7.4e-14, 4.7e-13 -> 4.6e-13, 7.0e-13 -> 6.9e-13, 1.65e-12 ->
+// 1.65e-12, Diels-Alder images 6.0e-13 -> 5.9e-13, 1.04e-12 -> 1.04e-12; in the
+// minimal basis, where a molecule of one H2O has nothing screened, 1.5e-16 ->
+// 1.1e-16, 8 H2O 6.7e-13 -> 6.7e-13 (DF_TAU_PRIM makes up for the rounding at the
+// default cutoffs). A caller who asks for a quartet cutoff below the default
+// kDfMinTau or a primitive cutoff below kDfMinPrim (the default is 1e-12 / 81 =
+// 1.23e-14) wants a smaller error than that rounding: everything in FP64 then.
+constexpr double kDfTau = 1e-2, kDfAll = 8796093022208.0 /* 2^43 */, kDfMinTau = 1e-12, kDfMinPrim = 1.2e-14;
 // The same for the gradient, whose bound Q_ab Q_cd |Gamma| carries no derivative
 // scale: the derivative integrals are up to some 1e2 times larger (2 sqrt(2
 // exponent)). Float-float minus FP64 gradient at one density and the same cutoffs
@@ -1016,7 +1021,7 @@ static int fock_build(pimd_ctx* ctx, Batch& bt, Mats& m, double tau, double fp32
         launch_to_float(M, Mf, bt.mtot, ctx->stream);
         ctx->stats.kernel_launches++;
     }
-    DfBuild df{df_bound(bt, df_tau, tau, tau_prim, tau, fp32_tau), 0, nullptr, ctx->boysd};
+    DfBuild df{df_bound(bt, df_tau, tau, tau_prim, tau, fp32_tau), tau * kDfAll, 0, nullptr, ctx->boysd};
     if (df.tau > 0.0) {
         dfloat* Md;
         ENSURE("Md", bt.mtot, Md);
@@ -1024,9 +1029,7 @@ static int fock_build(pimd_ctx* ctx, Batch& bt, Mats& m, double tau, double fp32
         ctx->stats.kernel_launches++;
         df.D = Md;
     }
-    // (a class with nothing left to FP64 is one launch, or two with FP32 quartets)
-    const auto jobs = class_jobs(
-        bt, [&](int cp) { return df.tau > 0.0 && class_pair_df(cp) && (!class_pair_df_all(cp) || fp32_tau > tau); });
+    const auto jobs = class_jobs(bt, [&](int cp) { return df.tau > 0.0 && class_pair_straight(cp); });
     const int rc = fan_out(ctx, (int)jobs.size(), [&](int k, cudaStream_t st) {
         const int cp = jobs[k].first;
         DfBuild d = df;
@@ -1574,7 +1577,7 @@ static int run_batch(pimd_ctx* ctx, int nrep, const int* natom_of, const int* Zc
         launch_shell_bounds(bt.S, bt.R, nrep, bt.maxsh, m.D, bt.Dsh, nullptr, ctx->stream);
         DfBuild df{df_bound(bt, kDfTauGrad, o->schwarz_tau, o->schwarz_tau * o->prim_screen, o->schwarz_tau * 1e-2,
                             o->fp32_tau),
-                   0, Md, ctx->boysd};
+                   0.0, 0, Md, ctx->boysd};
         if (df.tau > 0.0) {
             launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);
             ctx->stats.kernel_launches++;
@@ -1924,8 +1927,8 @@ extern "C" int pimd_autotune(pimd_ctx* ctx, int nrep, int natom, const int* Z, c
         cudaMemsetAsync(m.G, 0, sizeof(double) * bt.mtot, ctx->stream);
         launch_shell_bounds(bt.S, bt.R, bt.nrep, bt.maxsh, m.D, bt.Dsh, bt.R.active, ctx->stream);
         if (Mf) launch_to_float(m.D, Mf, bt.mtot, ctx->stream);
-        DfBuild df{df_bound(bt, kDfTau, o.schwarz_tau, o.schwarz_tau * o.prim_screen, o.schwarz_tau, o.fp32_tau), 0,
-                   nullptr, ctx->boysd};
+        DfBuild df{df_bound(bt, kDfTau, o.schwarz_tau, o.schwarz_tau * o.prim_screen, o.schwarz_tau, o.fp32_tau),
+                   o.schwarz_tau * kDfAll, 0, nullptr, ctx->boysd};
         dfloat* Md;
         if ((rc2 = dev_ensure(ctx, "Md", (size_t)bt.mtot, &Md))) break;
         launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);
@@ -1959,7 +1962,7 @@ extern "C" int pimd_autotune(pimd_ctx* ctx, int nrep, int natom, const int* Z, c
             launch_shell_bounds(bt.S, bt.R, nrep, bt.maxsh, m.D, bt.Dsh, nullptr, ctx->stream);
             DfBuild df{df_bound(bt, kDfTauGrad, o.schwarz_tau, o.schwarz_tau * o.prim_screen, o.schwarz_tau * 1e-2,
                                 o.fp32_tau),
-                       0, nullptr, ctx->boysd};
+                       0.0, 0, nullptr, ctx->boysd};
             dfloat* Md = nullptr;
             rc2 = dev_ensure(ctx, "Md", (size_t)bt.mtot, &Md);
             if (!rc2) launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);

@@ -137,6 +137,22 @@ def test_a_tighter_cutoff_of_either_kind_keeps_fp64(ctx, tau, prim, fp64):
     assert (launches(B) == launches(W)) == fp64
 
 
+@pytest.mark.parametrize("scale", [300.0, 1e6])
+def test_large_densities_leave_the_long_classes_to_fp64(ctx, scale):
+    """p and d shells of which nothing is screened and a density so large that
+    the cutoffs do not matter: what stays in float-floats is below 2^43 times the
+    cutoff, and the rounding below the 2^-46 of the norm that a build is allowed."""
+    sh = [inputs.Shell(2, [1.3, 0.5], [0.4, 0.7]), inputs.Shell(1, [0.8], [1.0])]
+    B, W = native.Basis({1: sh}), native.Basis({1: sh, 2: [inputs.Shell(0, [1e9], [1.0])]})
+    Z = np.array([1, 1], np.int32)
+    X = np.array([[[0.0, 0.0, 0.0], [0.2, 0.3, 1.6]]])
+    D = np.random.default_rng(3).normal(size=(1, B.nbf(Z), B.nbf(Z)))
+    D = scale * (D + D.transpose(0, 2, 1))
+    ref = _fock(ctx, W, Z, X, D, 0.0)
+    df, fp64 = [np.linalg.norm(_fock(ctx, b, Z, X, D) - ref) / np.linalg.norm(ref) for b in (B, W)]
+    assert df < fp64 + ROUNDING
+
+
 def _profiled(fn):
     """(fn(), kernels that ran on the device meanwhile)"""
     from torch.profiler import ProfilerActivity, profile
