@@ -45,7 +45,7 @@ struct pimd_basis {
     // flattened primitives (element-major, shell order) for the device
     std::vector<double> exps, coefs;
     std::vector<std::vector<int>> prim_off;  // per element, per shell
-    bool df_range = true;                    // exponents within the range of the float-float kernels
+    bool df_range = true;                    // within the range of the float-float kernels (df_in_range)
     long long uid = 0;                       // distinct per basis created in the process
 };
 
@@ -76,6 +76,22 @@ static void normalise(ShellDef& s)
             ov += c[i] * c[j] * pow(pi / p, 1.5) * dfact(2 * s.l - 1) / pow(2 * p, s.l);
         }
     for (int i = 0; i < s.nprim; i++) s.coefs[i] = c[i] / sqrt(ov);
+}
+
+// Whether a (normalised) shell is within the range of the float-float kernels:
+// its exponents, and what its coefficients make of the prefactors. A primitive
+// pair's is c0 c_a c_b exp(..) / (a + b), at most c0 w_a w_b with w = |c| / sqrt(2 a);
+// the product of two, the first number of every primitive quartet, is kept 8
+// decades below the largest FP32 number (tight d shells, and contractions of
+// nearly equal primitives with coefficients that nearly cancel, exceed it).
+static bool df_in_range(const ShellDef& s)
+{
+    const double c0 = sqrt(2.0) * pow(3.14159265358979323846, 1.25);
+    for (int i = 0; i < s.nprim; i++) {
+        const double w = fabs(s.coefs[i]) / sqrt(2.0 * s.exps[i]);
+        if (!(s.exps[i] > 1e-6 && s.exps[i] < 1e8 && c0 * c0 * w * w * w * w < 1e30)) return false;
+    }
+    return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -342,8 +358,8 @@ extern "C" int pimd_basis_create(pimd_basis** out, int nelem, const int* Z_of_el
                     return PIMD_EINVAL;
                 }
             }
-            for (int i = 0; i < d.nprim; i++) b->df_range = b->df_range && d.exps[i] > 1e-6 && d.exps[i] < 1e8;
             normalise(d);
+            b->df_range = b->df_range && df_in_range(d);
             offs.push_back((int)b->exps.size());
             for (int i = 0; i < d.nprim; i++) {
                 b->exps.push_back(d.exps[i]);

@@ -153,6 +153,23 @@ def test_large_densities_leave_the_long_classes_to_fp64(ctx, scale):
     assert df < fp64 + ROUNDING
 
 
+@pytest.mark.parametrize("coefs,exps", [([1.0, -0.999], [9e7, 8.9e7]), ([1.0], [9e7])])
+def test_large_prefactors_keep_fp64(ctx, coefs, exps):
+    """Tight p and d shells whose prefactors' products are outside FP32, with
+    coefficients that nearly cancel and without: the basis outside the range by
+    its exponents gives the same matrix, up to the order of the FP64 additions
+    (2^-46 of the norm)."""
+    sh = [inputs.Shell(2, exps, coefs), inputs.Shell(1, exps, coefs), inputs.Shell(0, [1.1], [1.0])]
+    B, W = native.Basis({1: sh}), native.Basis({1: sh, 2: [inputs.Shell(0, [1e9], [1.0])]})
+    Z = np.array([1, 1], np.int32)
+    X = np.array([[[0.0, 0.1, 0.0], [3e-4, -2e-4, 1e-4]]])
+    D = np.random.default_rng(4).normal(size=(1, B.nbf(Z), B.nbf(Z))) * 1e-9
+    D = D + D.transpose(0, 2, 1)
+    g, ref = [_fock(ctx, b, Z, X, D) for b in (B, W)]
+    assert np.isfinite(ref).all() and np.isfinite(g).all()
+    assert np.linalg.norm(g - ref) < ROUNDING * np.linalg.norm(ref)
+
+
 def _profiled(fn):
     """(fn(), kernels that ran on the device meanwhile)"""
     from torch.profiler import ProfilerActivity, profile
