@@ -58,9 +58,16 @@ static double dfact(int n)
     return r;
 }
 
+// overlap of primitives i and j of a shell without their coefficients (x^l
+// component): <g_a|g_b> = (pi/(a+b))^{3/2} (2l-1)!! / (2(a+b))^l
+static double self_overlap(const ShellDef& s, int i, int j)
+{
+    const double p = s.exps[i] + s.exps[j];
+    return pow(3.14159265358979323846 / p, 1.5) * dfact(2 * s.l - 1) / pow(2 * p, s.l);
+}
+
 // normalised contraction: primitive norm (2a/pi)^{3/4} (4a)^{l/2} / sqrt((2l-1)!!),
-// then the contraction scaled so that <phi|phi> = 1 for the x^l component,
-// <g_a|g_b> = (pi/(a+b))^{3/2} (2l-1)!! / (2(a+b))^l
+// then the contraction scaled so that <phi|phi> = 1 for the x^l component
 static void normalise(ShellDef& s)
 {
     const double pi = 3.14159265358979323846;
@@ -71,10 +78,7 @@ static void normalise(ShellDef& s)
     }
     double ov = 0.0;
     for (int i = 0; i < s.nprim; i++)
-        for (int j = 0; j < s.nprim; j++) {
-            const double p = s.exps[i] + s.exps[j];
-            ov += c[i] * c[j] * pow(pi / p, 1.5) * dfact(2 * s.l - 1) / pow(2 * p, s.l);
-        }
+        for (int j = 0; j < s.nprim; j++) ov += c[i] * c[j] * self_overlap(s, i, j);
     for (int i = 0; i < s.nprim; i++) s.coefs[i] = c[i] / sqrt(ov);
 }
 
@@ -83,9 +87,17 @@ static void normalise(ShellDef& s)
 // pair's is c0 c_a c_b exp(..) / (a + b), at most c0 w_a w_b with w = |c| / sqrt(2 a);
 // the product of two, the first number of every primitive quartet, is kept 8
 // decades below the largest FP32 number (tight d shells, and contractions of
-// nearly equal primitives with coefficients that nearly cancel, exceed it).
+// nearly equal primitives with coefficients that nearly cancel, exceed it). And a
+// contraction must not cancel by itself: the bounds that pick a quartet's
+// arithmetic are those of the contracted integrals, while the rounding is that of
+// the primitive ones, larger by up to the square of sum_ij |c_i c_j| S_ij (1
+// without signs, 1.1 to 1.5 in the usual contracted bases).
 static bool df_in_range(const ShellDef& s)
 {
+    double cancel = 0.0;
+    for (int i = 0; i < s.nprim; i++)
+        for (int j = 0; j < s.nprim; j++) cancel += fabs(s.coefs[i] * s.coefs[j]) * self_overlap(s, i, j);
+    if (!(cancel < 2.0)) return false;
     const double c0 = sqrt(2.0) * pow(3.14159265358979323846, 1.25);
     for (int i = 0; i < s.nprim; i++) {
         const double w = fabs(s.coefs[i]) / sqrt(2.0 * s.exps[i]);

@@ -170,6 +170,22 @@ def test_large_prefactors_keep_fp64(ctx, coefs, exps):
     assert np.linalg.norm(g - ref) < ROUNDING * np.linalg.norm(ref)
 
 
+@pytest.mark.parametrize("second", [-0.95, -0.7])
+def test_contractions_that_cancel_keep_fp64(ctx, second):
+    """Shells of two nearly equal primitives with coefficients of opposite sign:
+    the contracted integrals are 1e2 to 1e5 times smaller than the primitive ones,
+    and no further from exact than in FP64."""
+    sh = [inputs.Shell(l, [1.0, 0.9], [1.0, second]) for l in (2, 1, 0)]
+    B, W = native.Basis({1: sh}), native.Basis({1: sh, 2: [inputs.Shell(0, [1e9], [1.0])]})
+    Z = np.array([1, 1], np.int32)
+    X = np.array([[[0.0, 0.1, 0.0], [0.7, -0.5, 2.1]]])
+    D = np.random.default_rng(4).normal(size=(1, B.nbf(Z), B.nbf(Z))) * 1e-2
+    D = D + D.transpose(0, 2, 1)
+    ref = _fock(ctx, W, Z, X, D, 0.0)
+    df, fp64 = [np.linalg.norm(_fock(ctx, b, Z, X, D) - ref) / np.linalg.norm(ref) for b in (B, W)]
+    assert df < fp64 + ROUNDING
+
+
 def _profiled(fn):
     """(fn(), kernels that ran on the device meanwhile)"""
     from torch.profiler import ProfilerActivity, profile
