@@ -539,7 +539,10 @@ def main():
                               "flops_per_step": gflops / K, "ms_per_step": grad_ms / K,
                               "note": ("per executed primitive quartet: the generated recursion to order L + 1 with "
                                        "its four accumulated sets, set-up and Boys; the HRRs, the density "
-                                       "contraction and the Cartesian/spherical transforms are not counted")},
+                                       "contraction and the Cartesian/spherical transforms are not counted; peak "
+                                       "and frac are those of the FP64 pipe, which carries all classes above 900 "
+                                       "operations (nine tenths of the time); the others run mostly in "
+                                       "float-float arithmetic")},
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": int(coord_bytes),
                     "d2h_bytes_per_step": int(nrep * 8 + coord_bytes)},
             "gpu_launches": launches,

@@ -58,9 +58,9 @@ typedef struct {
     int diis_size;        /* 8 (Pulay subspace, 2..16) */
     double schwarz_tau;   /* 1e-12: quartets with Q_ab Q_cd below it are skipped (Sec. 3.1) */
     double fp32_tau;      /* 0: no FP32 quartets (all in FP64, or as float-floats, pairs of FP32
-                             numbers, whose rounding the default cutoffs outweigh; with a
-                             schwarz_tau below 1e-12, or schwarz_tau * prim_screen below 1.2e-14,
-                             all in FP64);
+                             numbers, where the rounding of a quartet stays below schwarz_tau;
+                             with schwarz_tau below 1e-12, or schwarz_tau * prim_screen below
+                             1.2e-14, all in FP64);
                              > schwarz_tau: quartets whose bound
                              Q_ab Q_cd max|D block| is below it (D: the density increment of an
                              incremental build) are evaluated in FP32 and accumulated in FP64 */

@@ -684,9 +684,12 @@ DF_ALL_MIN_FLOPS = 1000
 # float-float gradient kernel: up to this many operations per primitive quartet.
 # The gradient's recursion runs to order L + 1 into four accumulator sets, and
 # beyond this its code and registers outgrow the instruction caches and the
-# register file: one bead, FP64 -> float-float: (ps|ss) 8.5 -> 3.0 ms, (ps|ps)
-# 13.6 -> 4.9, (dp|ss), the largest in, 5.3 -> 4.3; (ds|ps), the smallest out,
-# 11.6 -> 11.7, (pp|ps) 24.1 -> 87.4.
+# register file. One (H2O)8 bead, each launch alone, FP64 -> scalar float-float
+# (the form that is built): (ps|ss) 8.5 -> 3.0 ms, (ps|ps) 13.6 -> 4.9, (dp|ss),
+# the largest in, 5.3 -> 4.3; (ds|ps), the smallest out, 11.6 -> 11.7, (pp|ps)
+# 24.1 -> 87.4. The packed form, on a slower GPU, (ds|ps) 15.8 -> 10.5, but (pp|ps)
+# 35.4 -> 42.3 and every other class above the limit slower: not built for the
+# one class.
 DF_GRAD_MAX_FLOPS = 900
 
 
