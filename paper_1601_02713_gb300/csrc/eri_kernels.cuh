@@ -217,7 +217,7 @@ __device__ __forceinline__ void prim_quartet(const dfloat (*sbra)[PIMD_MAXPP], i
 
 // rows of a kernel's shared bra data
 template <typename R>
-constexpr int bra_rows(int n) { return std::is_same<R, dfloat>::value ? (int)PP_NF : n; }
+constexpr int bra_rows(int n) { return std::is_same<R, dfloat>::value ? (int)PPD_NF : n; }
 
 __device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }

@@ -104,11 +104,12 @@ int launch_grad2e(int cp, const Pairs& P, const Shells& S, const Reps& R, const 
                    double tau_prim, double fxs, cudaStream_t st);
 void grad2e_tapes_upload();   // once per device
 void boys_table_upload(double** dev_tab, float** dev_tabf, dfloat** dev_tabd);
-// float-float copies: n values; the pairs' A - B vectors [3][npair]
+// float-float copies: n values; the pair data [PPD_NF][PIMD_MAXPP][npair] and the
+// pairs' A - B vectors [3][npair]
 void launch_to_dfloat(const double* src, dfloat* dst, long long n, cudaStream_t st);
 // *flag = 1 if some of the n values is above lim in magnitude or not a number, else 0
 void launch_any_above(const double* v, long long n, double lim, int* flag, cudaStream_t st);
-void launch_pair_vectors(const Pairs& P, const Shells& S, dfloat* abd, cudaStream_t st);
+void launch_pair_dfloat(const Pairs& P, const Shells& S, dfloat* ppd, dfloat* abd, cudaStream_t st);
 // FP32 copies for the mixed-precision quartets
 void launch_to_float(const double* src, float* dst, long long n, cudaStream_t st);
 

@@ -126,7 +126,7 @@ __global__ void pair_data_kernel(Pairs P, int* npp, double* pp, Shells S, BasisP
             const double Px = (ea * A[0] + eb * Bc[0]) * ip, Py = (ea * A[1] + eb * Bc[1]) * ip,
                          Pz = (ea * A[2] + eb * Bc[2]) * ip;
             const double vals[PP_NF] = {p,  Px, Py, Pz, c0 * kij, Px - A[0], Py - A[1], Pz - A[2],
-                                        0.5 * ip, 0.5 * ip * ip, ea, eb, Px - Bc[0], Py - Bc[1], Pz - Bc[2]};
+                                        0.5 * ip, 0.5 * ip * ip, ea, eb};
             for (int f = 0; f < PP_NF; f++) pp[((size_t)f * PIMD_MAXPP + k) * P.n + g] = vals[f];
             k++;
         }
@@ -576,17 +576,26 @@ void launch_any_above(const double* v, long long n, double lim, int* flag, cudaS
     any_above_kernel<<<1, 256, 0, st>>>(v, n, lim, flag);
 }
 
-__global__ void pair_vectors_kernel(Pairs P, Shells S, dfloat* abd)
+__global__ void pair_dfloat_kernel(Pairs P, Shells S, dfloat* ppd, dfloat* abd)
 {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= P.n) return;
-    for (int x = 0; x < 3; x++) abd[(size_t)x * P.n + g] = dfloat(S.xyz[3 * P.sa[g] + x] - S.xyz[3 * P.sb[g] + x]);
+    const size_t n = P.n;
+    const int sa = P.sa[g], sb = P.sb[g], np = P.npp[g];
+    for (int x = 0; x < 3; x++) abd[x * n + g] = dfloat(S.xyz[3 * sa + x] - S.xyz[3 * sb + x]);
+    for (int k = 0; k < np; k++) {
+        for (int f = 0; f < PP_NF; f++)
+            ppd[((size_t)f * PIMD_MAXPP + k) * n + g] = dfloat(P.pp[((size_t)f * PIMD_MAXPP + k) * n + g]);
+        for (int x = 0; x < 3; x++)
+            ppd[((size_t)(PP_PBX + x) * PIMD_MAXPP + k) * n + g] =
+                dfloat(P.pp[((size_t)(PP_PX + x) * PIMD_MAXPP + k) * n + g] - S.xyz[3 * sb + x]);
+    }
 }
 
-void launch_pair_vectors(const Pairs& P, const Shells& S, dfloat* abd, cudaStream_t st)
+void launch_pair_dfloat(const Pairs& P, const Shells& S, dfloat* ppd, dfloat* abd, cudaStream_t st)
 {
     if (P.n == 0) return;
-    pair_vectors_kernel<<<(P.n + 127) / 128, 128, 0, st>>>(P, S, abd);
+    pair_dfloat_kernel<<<(P.n + 127) / 128, 128, 0, st>>>(P, S, ppd, abd);
 }
 
 __global__ void to_float_kernel(const double* src, float* dst, long long n)

@@ -35,8 +35,9 @@ enum PPField {
     PP_O2P,               // 1 / (2p)
     PP_O2PP,              // 1 / (2p^2)
     PP_EA, PP_EB,         // exponents a, b (gradient weights)
-    PP_PBX, PP_PBY, PP_PBZ,  // P - B (float-float kernels)
-    PP_NF
+    PP_NF,
+    PP_PBX = PP_NF, PP_PBY, PP_PBZ,  // P - B: in the float-float copy alone
+    PPD_NF
 };
 constexpr int PP_NERI = PP_EA;
 
@@ -59,7 +60,7 @@ struct Pairs {
     const float* qp;      // qp[k * n + g]: Schwarz factor sqrt(max |(ij|ij)|) of primitive pair k alone
                           // (contraction coefficients included); the primitive pairs of every shell
                           // pair are stored in descending order of it
-    const dfloat* ppd;    // pp as float-floats
+    const dfloat* ppd;    // pp as float-floats, with P - B (like abd only where the call runs such kernels)
     const dfloat* abd;    // [3][n] A - B of the pair's shells (centre of sa minus centre of sb)
     const float* qg;      // qg[k * n + g] = qp_k 2 sqrt(2 max(a_k, b_k)): the scale of the derivative
                           // integrals of primitive pair k (d/dA of a Gaussian of exponent a ~ sqrt(2a))

@@ -121,6 +121,7 @@ struct pimd_ctx {
     float* boysf = nullptr;
     dfloat* boysd = nullptr;
     std::map<std::string, DevBuf> bufs;
+    bool df_live = false;   // the float-float copies belong to the running call
     std::string last_error;
     pimd_stats stats{};
     // MO cache keyed by replica index
@@ -176,6 +177,31 @@ static int set_err(pimd_ctx* ctx, int code, const std::string& msg)
             return set_err(ctx, PIMD_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
+// The float-float copies (df_prepare) take what device memory the rest of a call
+// leaves: outside the part of a call that reads them (df_live) they are given
+// back when an allocation needs the room.
+static bool df_release(pimd_ctx* ctx)
+{
+    bool any = false;
+    for (const char* name : {"ppd", "abd", "Md"}) {
+        DevBuf& b = ctx->bufs[name];
+        if (b.p) cudaFree(b.p);   // (waits for the device)
+        any = any || b.p;
+        b = DevBuf{};
+    }
+    return any;
+}
+static bool dev_malloc(pimd_ctx* ctx, void** p, size_t bytes)
+{
+    for (int attempt = 0; attempt < 2; attempt++) {
+        if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+        cudaGetLastError();
+        *p = nullptr;
+        if (ctx->df_live || !df_release(ctx)) break;
+    }
+    return false;
+}
+
 template <typename T>
 static int dev_ensure(pimd_ctx* ctx, const char* name, size_t count, T** out)
 {
@@ -185,10 +211,8 @@ static int dev_ensure(pimd_ctx* ctx, const char* name, size_t count, T** out)
         if (b.p) cudaFree(b.p);
         b.p = nullptr;
         b.cap = 0;
-        if (cudaMalloc(&b.p, bytes) != cudaSuccess) {
-            cudaGetLastError();
+        if (!dev_malloc(ctx, &b.p, bytes))
             return set_err(ctx, PIMD_ENOMEM, std::string("cudaMalloc failed for ") + name);
-        }
         b.cap = bytes;
     }
     *out = (T*)b.p;
@@ -459,7 +483,9 @@ extern "C" int pimd_last_stats(const pimd_ctx* ctx, pimd_stats* out)
 // ---------------------------------------------------------------------------
 struct Batch {
     int nrep = 0;
-    bool df_ok = false;         // float-float kernels allowed: exponents and coordinates within their range
+    bool df_range = false;      // basis and coordinates within the range of the float-float kernels
+    bool df_ok = false;         // ... and their copies made (df_prepare)
+    dfloat* Md = nullptr;       // the density as float-floats
     bool allow_odd = false;     // isolated atoms of the SAD guess (occupations set by the caller)
     std::vector<int> natom, atom0, nbf, nocc;
     std::vector<int> atom_f0;   // first function of each atom within its replica
@@ -513,6 +539,7 @@ static int class_pair_index(int X, int Y)
 static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, const int* Zc, const double* d_xyz,
                        const pimd_basis* basis, double tau, int split_size = 1, int split_rank = 0)
 {
+    ctx->df_live = false;   // an earlier call's float-float copies
     bt.nrep = nrep;
     bt.natom.assign(natom_of, natom_of + nrep);
     bt.atom0.resize(nrep + 1);
@@ -687,7 +714,7 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
         CK(cudaMemcpyAsync(npp.data(), d_npp, sizeof(int) * npair, cudaMemcpyDeviceToHost, ctx->stream));
     }
     CK(cudaStreamSynchronize(ctx->stream));
-    bt.df_ok = basis->df_range && !far;
+    bt.df_range = basis->df_range && !far;
     for (int q = 0; q < npair; q++)
         if (!isfinite(Q[q])) return set_err(ctx, PIMD_EINVAL, "non-finite integrals (check coordinates)");
     {
@@ -720,11 +747,7 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
         float *d_qp, *d_qg;
         ENSURE("qp", (size_t)PIMD_MAXPP * npair, d_qp);
         ENSURE("qg", (size_t)PIMD_MAXPP * npair, d_qg);
-        dfloat *d_ppd, *d_abd;
-        ENSURE("ppd", (size_t)PP_NF * PIMD_MAXPP * npair, d_ppd);
-        ENSURE("abd", (size_t)3 * npair, d_abd);
-        bt.P = Pairs{npair, d_pa, d_pb, d_npp, d_pp, d_Q, d_ppf, d_qp, d_ppd, d_abd, d_qg};
-        launch_pair_vectors(bt.P, bt.S, d_abd, ctx->stream);
+        bt.P = Pairs{npair, d_pa, d_pb, d_npp, d_pp, d_Q, d_ppf, d_qp, nullptr, nullptr, d_qg};
         launch_pair_data(bt.P, d_npp, d_pp, bt.S, bt.B, ctx->stream);
         // primitive-pair bounds, and each pair's primitives in descending order of them
         for (int X = 0; X < 6; X++) {
@@ -739,7 +762,6 @@ static int setup_batch(pimd_ctx* ctx, Batch& bt, int nrep, const int* natom_of, 
             ctx->stats.kernel_launches++;
         }
         launch_to_float(d_pp, d_ppf, (long long)PP_NF * PIMD_MAXPP * npair, ctx->stream);
-        launch_to_dfloat(d_pp, d_ppd, (long long)PP_NF * PIMD_MAXPP * npair, ctx->stream);
     }
     // quartet tiles: for bra pair i of class X and each run of ket pairs of
     // class Y <= X with equal primitive count, the ket pairs with
@@ -1023,14 +1045,35 @@ constexpr double kDfTau = 1e-2, kDfAll = 8796093022208.0 /* 2^43 */, kDfMinTau =
 // 9.3e-13 / 1.5e-13 / 1.4e-13, 8.7e-13; a Diels-Alder image 1.1e-12 / 7.3e-13 /
 // 3.9e-13, 2.2e-12. The gradient of 4 (H2O)8 beads takes 869 / 870 / 877 ms.
 constexpr double kDfTauGrad = 1e-4;
-// The bound below which a build with these cutoffs runs in float-floats, 0: none
-// (schwarz_tau, tau_prim: the caller's; tau: the kernels' quartet cutoff, in the
-// gradient a hundredth of schwarz_tau)
-static double df_bound(const Batch& bt, double df_tau, double schwarz_tau, double tau_prim, double tau,
-                       double fp32_tau)
+// The bound below which a build with the kernels' quartet cutoff tau runs in
+// float-floats, 0: none
+static double df_bound(const Batch& bt, double df_tau, double tau, double fp32_tau)
 {
-    return bt.df_ok && schwarz_tau >= kDfMinTau && tau_prim >= kDfMinPrim && df_tau > std::max(tau, fp32_tau) ? df_tau
-                                                                                                              : 0.0;
+    return bt.df_ok && df_tau > std::max(tau, fp32_tau) ? df_tau : 0.0;
+}
+
+// Makes the batch's float-float copies, after every other buffer of the call, where
+// its range and the caller's cutoffs allow float-floats; where device memory does
+// not hold them the call runs in FP64.
+static void df_prepare(pimd_ctx* ctx, Batch& bt, double schwarz_tau, double tau_prim)
+{
+    bt.df_ok = false;
+    if (!bt.df_range || !(schwarz_tau >= kDfMinTau && tau_prim >= kDfMinPrim)) return;
+    ctx->df_live = true;
+    const std::string err = ctx->last_error;
+    dfloat *ppd, *abd;
+    if (dev_ensure(ctx, "ppd", (size_t)PPD_NF * PIMD_MAXPP * bt.P.n, &ppd) ||
+        dev_ensure(ctx, "abd", (size_t)3 * bt.P.n, &abd) || dev_ensure(ctx, "Md", (size_t)bt.mtot, &bt.Md)) {
+        ctx->df_live = false;
+        df_release(ctx);
+        ctx->last_error = err;
+        return;
+    }
+    bt.P.ppd = ppd;
+    bt.P.abd = abd;
+    launch_pair_dfloat(bt.P, bt.S, ppd, abd, ctx->stream);
+    ctx->stats.kernel_launches++;
+    bt.df_ok = true;
 }
 
 // G' += G'(M) over all class pairs for the replicas in the active mask, with
@@ -1049,13 +1092,10 @@ static int fock_build(pimd_ctx* ctx, Batch& bt, Mats& m, double tau, double fp32
         launch_to_float(M, Mf, bt.mtot, ctx->stream);
         ctx->stats.kernel_launches++;
     }
-    DfBuild df{df_bound(bt, df_tau, tau, tau_prim, tau, fp32_tau), tau * kDfAll, 0, nullptr, ctx->boysd};
+    const DfBuild df{df_bound(bt, df_tau, tau, fp32_tau), tau * kDfAll, 0, bt.Md, ctx->boysd};
     if (df.tau > 0.0) {
-        dfloat* Md;
-        ENSURE("Md", bt.mtot, Md);
-        launch_to_dfloat(M, Md, bt.mtot, ctx->stream);
+        launch_to_dfloat(M, bt.Md, bt.mtot, ctx->stream);
         ctx->stats.kernel_launches++;
-        df.D = Md;
     }
     const auto jobs = class_jobs(bt, [&](int cp) { return df.tau > 0.0 && class_pair_straight(cp); });
     const int rc = fan_out(ctx, (int)jobs.size(), [&](int k, cudaStream_t st) {
@@ -1459,8 +1499,6 @@ static int run_batch(pimd_ctx* ctx, int nrep, const int* natom_of, const int* Zc
         float* Mf;
         ENSURE("Mf", bt.mtot, Mf);   // allocated before any capture
     }
-    dfloat* Md;
-    ENSURE("Md", bt.mtot, Md);
     double* Gsum = nullptr;   // force-split mode: G' summed over the processes
     if (split) ENSURE("Gsum", bt.mtot, Gsum);
     int *d_mode, *d_slot, *d_count, *d_on;
@@ -1468,6 +1506,7 @@ static int run_batch(pimd_ctx* ctx, int nrep, const int* natom_of, const int* Zc
     ENSURE("slot", nrep, d_slot);
     ENSURE("count", nrep, d_count);
     ENSURE("diis_on", nrep, d_on);
+    df_prepare(ctx, bt, o->schwarz_tau, o->schwarz_tau * o->prim_screen);
     for (int it = 1; it <= o->max_iter && nactive > 0; it++) {
         for (int r = 0; r < nrep; r++) mode[r] = active[r] ? mode[r] : 0;
         UPLOAD("mode", mode, d_mode);
@@ -1603,11 +1642,9 @@ static int run_batch(pimd_ctx* ctx, int nrep, const int* natom_of, const int* Zc
         }
         CK(cudaEventRecord(ctx->ev[4], ctx->stream));
         launch_shell_bounds(bt.S, bt.R, nrep, bt.maxsh, m.D, bt.Dsh, nullptr, ctx->stream);
-        DfBuild df{df_bound(bt, kDfTauGrad, o->schwarz_tau, o->schwarz_tau * o->prim_screen, o->schwarz_tau * 1e-2,
-                            o->fp32_tau),
-                   0.0, 0, Md, ctx->boysd};
+        const DfBuild df{df_bound(bt, kDfTauGrad, o->schwarz_tau * 1e-2, o->fp32_tau), 0.0, 0, bt.Md, ctx->boysd};
         if (df.tau > 0.0) {
-            launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);
+            launch_to_dfloat(m.D, bt.Md, bt.mtot, ctx->stream);
             ctx->stats.kernel_launches++;
         }
         const auto jobs = class_jobs(bt, [&](int cp) { return df.tau > 0.0 && grad_pair_df(cp) && ctx->grad_var[cp] == 1; });
@@ -1633,6 +1670,7 @@ static int run_batch(pimd_ctx* ctx, int nrep, const int* natom_of, const int* Zc
         }
     }
     // MO cache (and the final Fock matrix)
+    ctx->df_live = false;
     for (int r = 0; r < nrep; r++) {
         auto& mo = ctx->mo[r];
         const size_t bytes = sizeof(double) * bt.nbf[r] * bt.nbf[r];
@@ -1641,8 +1679,7 @@ static int run_batch(pimd_ctx* ctx, int nrep, const int* natom_of, const int* Zc
             if (b->p) cudaFree(b->p);
             b->p = nullptr;
             b->cap = 0;
-            if (cudaMalloc(&b->p, bytes) != cudaSuccess) {
-                cudaGetLastError();
+            if (!dev_malloc(ctx, &b->p, bytes)) {
                 mo.N = 0;
                 return set_err(ctx, PIMD_ENOMEM, "MO cache allocation failed");
             }
@@ -1918,6 +1955,7 @@ extern "C" int pimd_autotune(pimd_ctx* ctx, int nrep, int natom, const int* Z, c
         if ((r2 = sad_place(ctx, basis, bt, m, Zc.data(), active, m.D))) return r2;
         *Mf = nullptr;
         if (o.fp32_tau > o.schwarz_tau && (r2 = dev_ensure(ctx, "Mf", (size_t)bt.mtot, Mf))) return r2;
+        df_prepare(ctx, bt, o.schwarz_tau, o.schwarz_tau * o.prim_screen);
         return PIMD_OK;
     };
     auto timed = [&](std::vector<double>& out, int stride, int col, const std::vector<int>& use,
@@ -1955,12 +1993,8 @@ extern "C" int pimd_autotune(pimd_ctx* ctx, int nrep, int natom, const int* Z, c
         cudaMemsetAsync(m.G, 0, sizeof(double) * bt.mtot, ctx->stream);
         launch_shell_bounds(bt.S, bt.R, bt.nrep, bt.maxsh, m.D, bt.Dsh, bt.R.active, ctx->stream);
         if (Mf) launch_to_float(m.D, Mf, bt.mtot, ctx->stream);
-        DfBuild df{df_bound(bt, kDfTau, o.schwarz_tau, o.schwarz_tau * o.prim_screen, o.schwarz_tau, o.fp32_tau),
-                   o.schwarz_tau * kDfAll, 0, nullptr, ctx->boysd};
-        dfloat* Md;
-        if ((rc2 = dev_ensure(ctx, "Md", (size_t)bt.mtot, &Md))) break;
-        launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);
-        df.D = Md;
+        const DfBuild df{df_bound(bt, kDfTau, o.schwarz_tau, o.fp32_tau), o.schwarz_tau * kDfAll, 0, bt.Md, ctx->boysd};
+        if (bt.df_ok) launch_to_dfloat(m.D, bt.Md, bt.mtot, ctx->stream);
         rc2 = timed(ms, 4, ci, use, [&](int cp) {
             if (!bt.tiles[cp].empty())
                 launch_jk(cp, bt.P, bt.S, bt.R, bt.d_tiles[cp], (int)bt.tiles[cp].size(), m.D, Mf, df, m.G, ctx->boys,
@@ -1988,13 +2022,8 @@ extern "C" int pimd_autotune(pimd_ctx* ctx, int nrep, int natom, const int* Z, c
         if (!rc2) rc2 = dev_ensure(ctx, "tune_grad", (size_t)nrep * natom * 3, &d_g);
         if (!rc2) {
             launch_shell_bounds(bt.S, bt.R, nrep, bt.maxsh, m.D, bt.Dsh, nullptr, ctx->stream);
-            DfBuild df{df_bound(bt, kDfTauGrad, o.schwarz_tau, o.schwarz_tau * o.prim_screen, o.schwarz_tau * 1e-2,
-                                o.fp32_tau),
-                       0.0, 0, nullptr, ctx->boysd};
-            dfloat* Md = nullptr;
-            rc2 = dev_ensure(ctx, "Md", (size_t)bt.mtot, &Md);
-            if (!rc2) launch_to_dfloat(m.D, Md, bt.mtot, ctx->stream);
-            df.D = Md;
+            const DfBuild df{df_bound(bt, kDfTauGrad, o.schwarz_tau * 1e-2, o.fp32_tau), 0.0, 0, bt.Md, ctx->boysd};
+            if (bt.df_ok) launch_to_dfloat(m.D, bt.Md, bt.mtot, ctx->stream);
             for (int v = 0; v < 2 && !rc2; v++) {
                 std::vector<int> use(ncp, 0);
                 for (int cp = 0; cp < ncp; cp++)
@@ -2044,6 +2073,11 @@ extern "C" int pimd_fock_dev(pimd_ctx* ctx, int nrep, int natom, const int* Z, c
     {
         pimd_scf_opts d;
         pimd_scf_opts_default(&d);
+        if (fp32_tau > schwarz_tau) {
+            float* Mf;
+            ENSURE("Mf", bt.mtot, Mf);   // before what the float-float copies may take
+        }
+        df_prepare(ctx, bt, schwarz_tau, schwarz_tau * d.prim_screen);
         if ((rc = fock_build(ctx, bt, m, schwarz_tau, fp32_tau, m.D, schwarz_tau * d.prim_screen, 0.0))) return rc;
     }
     // G_out = G' + G'^T
