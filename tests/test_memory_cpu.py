@@ -1,7 +1,6 @@
 """Device memory of the float-float copies, without a GPU: the library linked to
 a stand-in runtime whose kernels do nothing and whose device holds a given number
 of bytes. The copies take only what the rest of a call leaves."""
-import glob
 import os
 import subprocess
 
@@ -136,9 +135,10 @@ def rows(tmp_path_factory):
     (tmp / "main.cpp").write_text(MAIN)
     cuda = os.path.dirname(os.path.dirname(build.nvcc_path()))
     exe = str(tmp / "main")
+    units = build.HAND_WRITTEN + [os.path.basename(u) for u in build.generate_sources()]
+    objs = [os.path.join(build.OBJ, u + ".o") for u in units]
     subprocess.run(["g++", "-std=c++17", "-w", "-I", os.path.join(cuda, "include"), "-I", build.INCLUDE,
-                    str(tmp / "main.cpp")] + sorted(glob.glob(os.path.join(build.OBJ, "*.o"))) + ["-o", exe],
-                   check=True)
+                    str(tmp / "main.cpp")] + objs + ["-o", exe], check=True)
     out = subprocess.run([exe], check=True, capture_output=True, text=True, timeout=300).stdout
     return [[int(x) for x in row.split()] for row in out.splitlines()]
 
